@@ -3,10 +3,9 @@
 // base with the randomized Hadamard or a dense random rotation), and fake quantization.
 //
 // Records are built by destination slot: after a slot -> token map (scatter_tok_kernel),
-// the affine kernel gives a warp 8 consecutive slots of one pool (lanes own half rows);
-// the rotated bases give a 128-thread CTA 64 slots (one thread per row, the whole row
-// in registers).  Either way a CTA's level count is uniform and its record writes are
-// contiguous.  The dense rotation runs its 128 x 128 product on tcgen05 instead.
+// the affine kernel gives a warp 4 consecutive slots of one pool (lanes own quarter rows),
+// the rotated bases 8 (two lanes per row, half a row in registers).  Either way the level
+// count is uniform and the record writes are contiguous.  The dense rotation runs its 128 x 128 product on tcgen05 instead.
 //
 // Arithmetic (binary32, round to nearest even, no contraction), per row x:
 //  affine: s = fp16((max-min)/(L-1)) limited to 65504, z = fp16(min);
@@ -65,46 +64,10 @@ __device__ __forceinline__ void put_bits(uint32_t (&w)[3], int pos, int n, uint3
   if (sh + n > 32) w[wd + 1] |= v >> (32 - sh);
 }
 
-// The bit field of one quarter from its 32 rounded values: m[j] is the bit pattern of
-// 1.5 * 2^23 + c_j, so sums of L-weighted patterns give the radix value t modulo 2^32
-// once the weighted 1.5 * 2^23 terms are taken off.
-template <int L>
-__device__ __forceinline__ void quarter_field(const uint32_t (&m)[32], uint32_t (&w)[3]) {
-  using F = Fmt<L>;
-  constexpr uint32_t kMagic = 0x4B400000u;
-  w[0] = w[1] = w[2] = 0u;
-  if constexpr (F::G == 1 && F::LG == (1u << F::W)) {
-    // L = 2, 4, 8: ceil(c 2^W / L) = c, each code its own W-bit symbol
-#pragma unroll
-    for (int sy = 0; sy < 32; ++sy) put_bits(w, sy * F::W, F::W, m[sy] - kMagic);
-  } else {
-#pragma unroll
-    for (int sy = 0; sy < F::NG; ++sy) {
-      uint32_t t = 0, wsum = 0;
-#pragma unroll
-      for (int k = 0; k < F::G; ++k) {
-        t = t * (uint32_t)L + m[sy * F::G + k];
-        wsum = wsum * (uint32_t)L + 1u;
-      }
-      t -= wsum * kMagic;
-      put_bits(w, sy * F::W, F::W, ((t << F::W) + F::LG - 1u) / F::LG);
-    }
-    if constexpr (F::R > 0) {
-      uint32_t t = 0, wsum = 0;
-#pragma unroll
-      for (int k = 0; k < F::R; ++k) {
-        t = t * (uint32_t)L + m[32 - F::R + k];
-        wsum = wsum * (uint32_t)L + 1u;
-      }
-      t -= wsum * kMagic;
-      put_bits(w, F::NG * F::W, F::WT, ((t << F::WT) + F::LR - 1u) / F::LR);
-    }
-  }
-}
-
 // One code of a quarter's field, streamed in order (j = 0..31, compile-time after
 // unrolling): m is the magic-number pattern 1.5 * 2^23 + c_j, t the running radix value
-// of the open symbol; each completed symbol's beta goes into the field, as quarter_field.
+// of the open symbol (sums of L-weighted patterns give it modulo 2^32 once the weighted
+// 1.5 * 2^23 terms are taken off); each completed symbol's beta goes into the field.
 template <int L>
 __device__ __forceinline__ void field_push(uint32_t (&w)[3], uint32_t& t, int j, uint32_t m) {
   using F = Fmt<L>;
@@ -257,29 +220,29 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kAffineCtas)
 }
 
 // ------------------------------ rotated bases by slot, two threads per row -----
-// TQ and rotated affine records built by destination slot, as for the affine base: a
-// CTA of 256 threads takes 64 consecutive slots of one pool of one (sequence, layer,
-// KV head), so the level count is uniform.  Thread tid holds half f = tid & 1 (dims
-// 64f .. 64f + 63, quarters 2f and 2f + 1) of row tid >> 1 of the block (K of slot
-// tid >> 2 when bit 1 of tid is 0, V when it is 1), in registers as 32 packed pairs
+// TQ and rotated affine records built by destination slot, as for the affine base: a warp
+// takes tiles of 8 consecutive slots of one pool of one (sequence, layer, KV head), so the
+// level count is uniform.  Lane 4i + 2r + f holds half f (dims 64f .. 64f + 63, quarters
+// 2f and 2f + 1) of row r (0 = K, 1 = V) of slot i, in registers as 32 packed pairs
 // (x_j, x_{j+32}).  The Walsh-Hadamard butterflies run in the quantizer's stage order
 // (the same roundings as any other evaluation of them): stages 1..16 as packed
 // operations across pairs, stage 32 inside each pair, stage 64 with the partner lane.
 // Then the norm or the min/max (combined across the two halves), the codes, the two
-// quarters' bit fields; the threads then assemble the block's record words from the
-// rows' bit images and write them in order with 4-byte stores.
+// quarters' bit fields; each lane puts its half's bits into the tile's record image, which
+// leaves in order with 16-byte stores.
 constexpr int kRowSlots = 64;
 constexpr int kRowStride = 272;  // bytes per staged row: 256 + 16 spreads the banks
-constexpr int kRowBitWords = 13;  // words per row's bit image (12 used at most)
+constexpr int kTileSlots = 8;    // slots of a warp's tile
 constexpr int kRows2Threads = 256;
 constexpr int kHalfStride = 144;  // bytes per half-row slot: 128 + 16 (9 x 16 B: the 8 lanes
                                   // of a quarter warp reach distinct banks)
 constexpr int kRows2StageBytes = kRows2Threads * kHalfStride;
-// resident CTAs per SM (80 registers a thread).  The TQ path at 4 and more levels keeps
-// its packed thresholds in registers too and spills a few words at this budget; it still
-// ran 6% faster than at 2 CTAs per SM (128 registers, no spills).
-constexpr int rows2_ctas(int) { return 3; }
-static_assert(kRowBitWords + 1 <= kHalfStride / 4, "bit image and parameters fit a half slot");
+constexpr int kWarpStageBytes = 32 * kHalfStride;
+// The quantizer: CTAs of 128 threads, 5 per SM (96 registers, 20 warps).  At 6 per SM (80
+// registers) the pairs spill and at 4 fewer warps hide the shuffles: the 3 x 20011 rotated
+// prompt took 159 us at 5, 166 at 24 warps, 182 at 16.
+constexpr int kRowsThreads = 128;
+constexpr int kRowsCtas = 5;
 
 // packed binary32 pairs (two independent IEEE operations, rounded to nearest)
 __device__ __forceinline__ unsigned long long f2_add(unsigned long long a, unsigned long long b) {
@@ -328,6 +291,19 @@ __device__ __forceinline__ unsigned long long f2_fma(unsigned long long a, unsig
   return d;
 }
 
+// a * b in a form that is not fused into the operation that takes the result: a * b + -0
+// is the rounded product, signed zeros included.  nz must reach the code generator as a
+// run-time value (opaque_neg_zero): it turns a constant -0 back into a multiply, and fuses.
+__device__ __forceinline__ unsigned long long f2_mul_only(unsigned long long a, unsigned long long b,
+                                                          unsigned long long nz) {
+  return f2_fma(a, b, nz);
+}
+__device__ __forceinline__ unsigned long long opaque_neg_zero(uint32_t* scratch) {
+  *reinterpret_cast<volatile uint32_t*>(scratch) = 0x80000000u;
+  const uint32_t z = *reinterpret_cast<volatile uint32_t*>(scratch);
+  return (unsigned long long)z | ((unsigned long long)z << 32);
+}
+
 // Butterfly stages 1, 2, 4, 8, 16 and 32 of the row transform over one half of the row,
 // held as packed pairs xp[j] = (x_j, x_{j+32}) (half-local indices): stages 1..16 pair
 // registers j and j + hs and so run packed, stage 32 works inside each register.  Each
@@ -350,40 +326,6 @@ __device__ __forceinline__ void fwht_half(unsigned long long (&xp)[32]) {
   }
 }
 
-// The bit field of one quarter from its 32 codes c_j = m[j] - kOff (kOff: 1.5 * 2^23 for
-// magic-number patterns, 0 for plain codes), as quarter_field.
-template <int L, uint32_t kOff>
-__device__ __forceinline__ void quarter_field_off(const uint32_t (&m)[32], uint32_t (&w)[3]) {
-  using F = Fmt<L>;
-  w[0] = w[1] = w[2] = 0u;
-  if constexpr (F::G == 1 && F::LG == (1u << F::W)) {
-#pragma unroll
-    for (int sy = 0; sy < 32; ++sy) put_bits(w, sy * F::W, F::W, m[sy] - kOff);
-  } else {
-#pragma unroll
-    for (int sy = 0; sy < F::NG; ++sy) {
-      uint32_t t = 0, wsum = 0;
-#pragma unroll
-      for (int k = 0; k < F::G; ++k) {
-        t = t * (uint32_t)L + m[sy * F::G + k];
-        wsum = wsum * (uint32_t)L + 1u;
-      }
-      t -= wsum * kOff;
-      put_bits(w, sy * F::W, F::W, ((t << F::W) + F::LG - 1u) / F::LG);
-    }
-    if constexpr (F::R > 0) {
-      uint32_t t = 0, wsum = 0;
-#pragma unroll
-      for (int k = 0; k < F::R; ++k) {
-        t = t * (uint32_t)L + m[32 - F::R + k];
-        wsum = wsum * (uint32_t)L + 1u;
-      }
-      t -= wsum * kOff;
-      put_bits(w, F::NG * F::W, F::WT, ((t << F::WT) + F::LR - 1u) / F::LR);
-    }
-  }
-}
-
 // TQ codes of both quarters of a half, straight into their bit fields.  u2[j] holds the
 // pair (u of quarter 0, u of quarter 1) at dim j of the quarters; t2[k] the pair
 // (thr_k, thr_k), ascending, with a zero threshold taken as +0.  d = thr_k - u rounds to
@@ -393,7 +335,7 @@ __device__ __forceinline__ void quarter_field_off(const uint32_t (&m)[32], uint3
 //   L = 2, 4, 8: the code's binary digits from those bits (parities and middles of the
 //   thermometer), shifted into the field most significant bit first, one funnel shift
 //   per bit (code j occupies bits jW .. jW + W - 1 of the field);
-//   other L: c as a sum of the bits, radix groups as quarter_field.
+//   other L: c as a sum of the bits, radix groups as field_push.
 template <int L>
 __device__ __forceinline__ void tq_fields(const unsigned long long (&u2)[32],
                                           const unsigned long long (&t2)[7],
@@ -439,7 +381,7 @@ __device__ __forceinline__ void tq_fields(const unsigned long long (&u2)[32],
       }
     }
   } else {
-    // c = sum of the comparison bits; symbols beta = ceil(t 2^W / L^G) as quarter_field
+    // c = sum of the comparison bits; symbols beta = ceil(t 2^W / L^G)
     auto code = [&](int j, uint32_t& cl, uint32_t& ch) {
       cl = 0u; ch = 0u;
 #pragma unroll
@@ -477,28 +419,23 @@ __device__ __forceinline__ void tq_fields(const unsigned long long (&u2)[32],
   }
 }
 
-// One half of every row of a 64-slot block (see above).  stage: the block's half-row
-// slots (thread tid's 128 bytes at tid * kHalfStride); smask: the (layer, head)'s sign
-// masks, one word per fp16 pair of dims (0x8000 in a half whose sign is -1).
-template <int BASE, int L>
-__device__ void rows_half(const QuantArgs& a, int b, int l, int h, bool hi, int64_t s0,
-                          int nslots, uint8_t* stage, const uint32_t* smask) {
-  using F = Fmt<L>;
-  constexpr int kWords = (4 * F::QB + 31) / 32;
-  constexpr int kRecW = (2 * F::RB + (BASE == SEMKV_BASE_TQ ? 4 : 8)) / 4;
-  constexpr int kSh = (2 * F::QB) & 31;        // bit offset of half 1 in its first word
-  constexpr int kWb = (2 * F::QB) >> 5;        // that word
-  constexpr int kW0 = (2 * F::QB + 31) / 32;   // words half 0 touches
-  constexpr int kW1 = (kSh + 2 * F::QB + 31) / 32;  // words half 1 touches, from kWb
-  static_assert(kWords <= 12 && F::QB <= 96 && kW1 <= 7, "row image size");
-  const int tid = threadIdx.x, f = tid & 1;
-  const int64_t cap = hi ? a.hi_cap : a.lo_cap;
-  const int64_t pbase = hi ? a.hi_base : a.lo_base;
-  const int64_t bh = ((int64_t)b * a.NL + l) * a.H + h;
+// One tile: 8 slots of one pool, the warp's lanes 4i .. 4i + 3 on slot i (K dims 0..63, K
+// dims 64..127, V likewise), in two parts so that the first is compiled once for all level
+// counts: the body is straight-line code of several hundred instructions, and two copies of
+// it in use at once do not stay in the instruction cache.
+//
+// rows_front: the rotated half row as pairs (u for the rotated affine base, w for TQ) and
+// the row's parameters.  stage: the lane's 128 bytes at lane * kHalfStride; smask: the
+// (layer, head)'s sign masks, one word per fp16 pair of dims (0x8000 in a half whose sign
+// is -1).
+template <int BASE>
+__device__ __forceinline__ void rows_front(int L, const uint8_t* stage, const uint32_t* smask,
+                                           unsigned long long nz, unsigned long long (&xp)[32],
+                                           uint32_t& param, float& invq, float& zq, bool& live) {
+  const int lane = threadIdx.x & 31, f = lane & 1;
   // ---- the half, sign-flipped on its fp16 bits (the signs are +-1), as pairs
-  unsigned long long xp[32];
-  if ((tid >> 2) < nslots) {
-    const uint4* src = reinterpret_cast<const uint4*>(stage + tid * kHalfStride);
+  {
+    const uint4* src = reinterpret_cast<const uint4*>(stage + lane * kHalfStride);
     const uint4* msk = reinterpret_cast<const uint4*>(smask + 32 * f);
     uint32_t wv[32];
 #pragma unroll
@@ -513,14 +450,7 @@ __device__ void rows_half(const QuantArgs& a, int b, int l, int h, bool hi, int6
       const int sh = 16 * (j & 1);
       xp[j] = f2_pack(f16_to_f32((uint16_t)(lo >> sh)), f16_to_f32((uint16_t)(hi2 >> sh)));
     }
-  } else {
-#pragma unroll
-    for (int j = 0; j < 32; ++j) xp[j] = 0ull;
   }
-  uint32_t param;
-  float invq;  // TQ: 1/n;  affine: 1/s
-  float zq = 0.0f;
-  bool live;
   if constexpr (BASE == SEMKV_BASE_TQ) {
     // the norm's fixed tree: 32 in-order partials of 4 squares (this half holds partials
     // 16f + g in the low lanes, 16f + g + 8 in the high ones), then the pairwise stages
@@ -565,9 +495,10 @@ __device__ void rows_half(const QuantArgs& a, int b, int l, int h, bool hi, int6
   }
   if constexpr (BASE == SEMKV_BASE_AFFINE_HAD) {
     float mn = INFINITY, mx = -INFINITY;
+    const unsigned long long rs2 = f2_pack(kInvSqrtD, kInvSqrtD);
 #pragma unroll
     for (int j = 0; j < 32; ++j) {
-      xp[j] = f2_pack(__fmul_rn(f2_lo(xp[j]), kInvSqrtD), __fmul_rn(f2_hi(xp[j]), kInvSqrtD));
+      xp[j] = f2_mul_only(xp[j], rs2, nz);
       mn = fminf(mn, fminf(f2_lo(xp[j]), f2_hi(xp[j])));
       mx = fmaxf(mx, fmaxf(f2_lo(xp[j]), f2_hi(xp[j])));
     }
@@ -586,96 +517,113 @@ __device__ void rows_half(const QuantArgs& a, int b, int l, int h, bool hi, int6
     invq = live ? __fdiv_rn(1.0f, sv) : 0.0f;
     param = (uint32_t)s16 | ((uint32_t)z16 << 16);
   }
+}
+
+// rows_back: the codes, the record image in the stage and the records (rec: the first one
+// in the pool).
+template <int BASE, int L>
+__device__ __forceinline__ void rows_back(const float* thr, uint8_t* stage, uint8_t* rec, int ns,
+                                          unsigned long long nz, unsigned long long (&xp)[32],
+                                          uint32_t param, float invq, float zq, bool live) {
+  using F = Fmt<L>;
+  constexpr int kRecW = (2 * F::RB + (BASE == SEMKV_BASE_TQ ? 4 : 8)) / 4;
+  constexpr int kBits = 2 * F::QB;             // a half's bits
+  constexpr int kW0 = (kBits + 31) / 32;
+  static_assert(F::QB <= 96 && 8 * kRecW * 4 <= 32 * kHalfStride, "the image fits the stage");
+  const int lane = threadIdx.x & 31, f = lane & 1;
+  const bool active = (lane >> 2) < ns;
   // ---- codes, quarter 2f from the low lanes, then quarter 2f + 1 from the high ones
-  uint32_t lw[7];
+  uint32_t lw[kW0];
 #pragma unroll
-  for (int k = 0; k < 7; ++k) lw[k] = 0u;
-  const unsigned long long inv2 = f2_pack(invq, invq);
+  for (int k = 0; k < kW0; ++k) lw[k] = 0u;
   if constexpr (BASE == SEMKV_BASE_TQ) {
     // c = #{k : u > thr_k} (ties go low); a zero-norm row compares against +inf
-    const float* tg = hi ? a.thr_hi : a.thr_lo;
     unsigned long long t2[7];
 #pragma unroll
     for (int k = 0; k < L - 1; ++k) {
-      const float tk = live ? __fadd_rn(__ldg(tg + k), 0.0f) : INFINITY;
+      const float tk = live ? thr[k] : INFINITY;
       t2[k] = f2_pack(tk, tk);
     }
     // u = y * fl(1/n), rounded before the comparisons subtract it
+    const unsigned long long inv2 = f2_pack(invq, invq);
 #pragma unroll
-    for (int j = 0; j < 32; ++j) xp[j] = f2_pack(__fmul_rn(f2_lo(xp[j]), invq), __fmul_rn(f2_hi(xp[j]), invq));
+    for (int j = 0; j < 32; ++j) xp[j] = f2_mul_only(xp[j], inv2, nz);
     uint32_t fw0[3], fw1[3];
     tq_fields<L>(xp, t2, fw0, fw1);
-    or_field<7>(lw, 0, fw0);
-    or_field<7>(lw, F::QB, fw1);
+    or_field<kW0>(lw, 0, fw0);
+    or_field<kW0>(lw, F::QB, fw1);
   } else {
     // rint(clamp((u - z) / s)) = clamp(rint(...)) for integer bounds; + 1.5 * 2^23 rounds
     // to nearest even and leaves the code in the low bits of the pattern
-    const unsigned long long z2 = f2_pack(zq, zq);
+    const unsigned long long z2 = f2_pack(zq, zq), inv2 = f2_pack(invq, invq);
     const unsigned long long mg2 = f2_pack(12582912.0f, 12582912.0f);
+    // Neither bound can be reached when z was not limited (u >= z) and s is a normal fp16
+    // value that was not limited either: s is then within 2^-11 of (max u - z) / (L - 1),
+    // so (u - z) / s < L - 1/2.  NaN rows and s = 0 fail the test.
+    const float sv = f16_to_f32((uint16_t)(param & 0xFFFFu));
+    const bool plain = zq > -65504.0f && sv >= 0x1p-14f && sv < 65504.0f;
+#pragma unroll
+    for (int j = 0; j < 32; ++j) xp[j] = f2_mul_only(f2_sub(xp[j], z2), inv2, nz);
+    if (!__all_sync(0xffffffffu, plain || !active)) {
+#pragma unroll
+      for (int j = 0; j < 32; ++j)
+        xp[j] = f2_pack(fminf(fmaxf(f2_lo(xp[j]), 0.0f), (float)(L - 1)),
+                        fminf(fmaxf(f2_hi(xp[j]), 0.0f), (float)(L - 1)));
+    }
+    uint32_t w0[3] = {0u, 0u, 0u}, w1[3] = {0u, 0u, 0u}, t0 = 0u, t1 = 0u;
 #pragma unroll
     for (int j = 0; j < 32; ++j) {
-      const unsigned long long d = f2_mul(f2_sub(xp[j], z2), inv2);
-      const float ylo = fminf(fmaxf(f2_lo(d), 0.0f), (float)(L - 1));
-      const float yhi = fminf(fmaxf(f2_hi(d), 0.0f), (float)(L - 1));
-      xp[j] = f2_add(f2_pack(ylo, yhi), mg2);
+      const unsigned long long y = f2_add(xp[j], mg2);
+      field_push<L>(w0, t0, j, (uint32_t)y);
+      field_push<L>(w1, t1, j, (uint32_t)(y >> 32));
     }
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      uint32_t m[32];
-#pragma unroll
-      for (int j = 0; j < 32; ++j) m[j] = __float_as_uint(q ? f2_hi(xp[j]) : f2_lo(xp[j]));
-      uint32_t fw[3];
-      quarter_field_off<L, 0x4B400000u>(m, fw);
-      or_field<7>(lw, q * F::QB, fw);
-    }
+    or_field<kW0>(lw, 0, w0);
+    or_field<kW0>(lw, F::QB, w1);
   }
-  // ---- the row's bit image and parameters, in half 0's slot: half 0 writes words
-  // 0..kWb (word kWb with half 1's low bits when half 1 starts inside it), half 1 the rest
-  uint32_t* img = reinterpret_cast<uint32_t*>(stage + (tid & ~1) * kHalfStride);
-  if constexpr (kSh != 0) {
+  // ---- the record image.  A half starts at bit `off` of its record; the word it shares
+  // with the next half (the next lane) takes that half's first word, which then is not
+  // written again.
+  constexpr int kSpan = (31 + kBits + 31) / 32;  // words a half touches at most
+  const int q = lane & 3;
+  const int off = (q >> 1) * 8 * F::RB + f * kBits;
+  const int wd0 = off >> 5, sh = off & 31;
+  const int cnt = ((off + kBits + 31) >> 5) - wd0;
+  const int next = q == 0 ? kBits : q == 1 ? 8 * F::RB : q == 2 ? 8 * F::RB + kBits : 16 * F::RB;
+  const bool share_next = (next >> 5) < wd0 + cnt;
+  const int prev_end = q == 0 ? -1 : q == 1 ? kBits - 1 : q == 2 ? 2 * kBits - 1 : 8 * F::RB + kBits - 1;
+  const bool share_prev = (prev_end >> 5) == wd0 && q != 0;
+  uint32_t v[kSpan];
 #pragma unroll
-    for (int k = kW1 - 1; k >= 0; --k) {
-      const uint32_t v = (lw[k] << kSh) | (k > 0 ? lw[k - 1] >> (32 - kSh) : 0u);
-      if (f) lw[k] = v;
-    }
-  }
-  const uint32_t first1 = __shfl_xor_sync(0xffffffffu, lw[0], 1);
-  __syncwarp();  // both halves' values were read from the slots
-  if ((tid >> 2) < nslots) {
+  for (int k = 0; k < kSpan; ++k)
+    v[k] = __funnelshift_l(k > 0 && k - 1 < kW0 ? lw[k - 1] : 0u, k < kW0 ? lw[k] : 0u, sh);
+  const uint32_t first = __shfl_down_sync(0xffffffffu, v[0], 1);
+#pragma unroll
+  for (int k = kBits / 32 > 0 ? kBits / 32 - 1 : 0; k < kSpan; ++k)
+    v[k] |= (share_next && k == cnt - 1) ? first : 0u;
+  uint32_t* img = reinterpret_cast<uint32_t*>(stage);
+  __syncwarp();  // every half row has been read
+  if (active) {
+    uint32_t* r = img + (lane >> 2) * kRecW;
+#pragma unroll
+    for (int k = 0; k < kSpan; ++k)
+      if (k < cnt && (k > 0 || !share_prev)) r[wd0 + k] = v[k];
     if (f == 0) {
-#pragma unroll
-      for (int k = 0; k < kW0; ++k) img[k] = (kSh != 0 && k == kWb) ? (lw[k] | first1) : lw[k];
-      img[kRowBitWords] = param;
-    } else {
-#pragma unroll
-      for (int k = (kSh != 0 ? 1 : 0); k < kW1; ++k) img[kWb + k] = lw[k];
+      if constexpr (BASE == SEMKV_BASE_TQ)
+        reinterpret_cast<uint16_t*>(r + (2 * F::RB) / 4)[q >> 1] = (uint16_t)param;
+      else
+        r[(2 * F::RB) / 4 + (q >> 1)] = param;
     }
   }
-  // ---- records: slot i's two rows are threads 4i .. 4i + 3, so each warp assembles its
-  // own 8 slots' records (contiguous words, one 4-byte word per lane and step)
   __syncwarp();
-  const int warp = tid >> 5, lane = tid & 31;
-  const int ns = min(8, nslots - 8 * warp);
-  uint32_t* recs = reinterpret_cast<uint32_t*>(hi ? a.hi_pool : a.lo_pool) +
-                   (bh * cap + pbase + s0 + 8 * warp) * kRecW;
-  for (int wi = lane; wi < ns * kRecW; wi += 32) {
-    const int i = 8 * warp + wi / kRecW, j = wi - (wi / kRecW) * kRecW;
-    const uint32_t* K = reinterpret_cast<const uint32_t*>(stage + (4 * i) * kHalfStride);
-    const uint32_t* V = reinterpret_cast<const uint32_t*>(stage + (4 * i + 2) * kHalfStride);
-    uint32_t word;
-    if (4 * j >= 2 * F::RB) {
-      const int pj = j - (2 * F::RB) / 4;
-      if constexpr (BASE == SEMKV_BASE_TQ) word = K[kRowBitWords] | (V[kRowBitWords] << 16);
-      else word = pj ? V[kRowBitWords] : K[kRowBitWords];
-    } else if (4 * j + 4 <= F::RB) {
-      word = K[j];
-    } else {
-      const int vb = 4 * j - F::RB;  // byte of the V row at this word's first byte
-      if (vb >= 0) word = __funnelshift_r(V[vb >> 2], V[(vb >> 2) + 1], 8 * (vb & 3));
-      else word = K[j] | (V[0] << (8 * -vb));
-    }
-    recs[wi] = word;
+  // ---- the records are contiguous: 16 bytes per lane where the pool position allows
+  const int words = ns * kRecW;
+  int done = 0;
+  if ((reinterpret_cast<uintptr_t>(rec) & 15u) == 0) {
+    for (int i = lane; i < words / 4; i += 32)
+      reinterpret_cast<uint4*>(rec)[i] = reinterpret_cast<const uint4*>(img)[i];
+    done = words & ~3;
   }
+  for (int i = done + lane; i < words; i += 32) reinterpret_cast<uint32_t*>(rec)[i] = img[i];
 }
 
 // ---- shared addresses and mbarriers
@@ -685,28 +633,6 @@ __device__ __forceinline__ uint32_t dsmem_u32(const void* p) {
 __device__ __forceinline__ void dbar_init(uint64_t* bar) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(dsmem_u32(bar)) : "memory");
 }
-// block t of the pass, decoded once: (sequence, layer, KV head), pool, first slot and
-// slot count (32-bit arithmetic: the launcher keeps the block count below 2^31)
-struct RowsTile {
-  int b, l, h;
-  bool hi;
-  int s0, nslots;
-};
-__device__ __forceinline__ RowsTile rows_tile(uint32_t t, uint32_t nb_hi, uint32_t per_bh,
-                                              uint32_t n_hi, uint32_t n_lo, uint32_t H,
-                                              uint32_t NL) {
-  RowsTile x;
-  const uint32_t bhi = t / per_bh, r = t - bhi * per_bh;
-  x.hi = r < nb_hi;
-  x.s0 = (int)((x.hi ? r : r - nb_hi) * kRowSlots);
-  x.nslots = min(kRowSlots, (int)(x.hi ? n_hi : n_lo) - x.s0);
-  const uint32_t q = bhi / H;
-  x.h = (int)(bhi - q * H);
-  x.b = (int)(q / NL);
-  x.l = (int)(q - (uint32_t)x.b * NL);
-  return x;
-}
-
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dsmem_u32(dst)), "l"(src) : "memory");
 }
@@ -718,71 +644,143 @@ __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-// Persistent CTAs of 256 threads over the blocks (64 slots of one pool of one (sequence,
-// layer, KV head)), in a two-stage pipeline: while a block is quantized, the halves of
-// the CTA's next block are already on their way.  Thread tid brings half tid & 1 of its
-// row into its own slot of the stage with eight 16-byte cp.async copies (one commit
-// group per block), and the first 64 threads write the next block's sign masks; a
-// thread waits for its own group, then the CTA barrier (the only one per block)
-// publishes the stage.
+// A position in the tiles: tile r of (sequence, layer, head) bhi, the high pool's tiles
+// before the low one's.
+struct RowsPos {
+  uint32_t bhi, r;
+};
+// Warps over tiles of 8 slots: a CTA takes a contiguous range, its warps the tiles in turn,
+// each warp with its own two-stage pipeline.  While a tile is quantized, the next one's half
+// rows (8 cp.async of 16 bytes per lane into the lane's slot) and the one after's token
+// indices are on their way.  No warp waits for another, and the positions stay in uniform
+// registers (they leave room for the pairs, which otherwise spill).
+//
+// Bound by instruction issue: 76 (rotated affine) and 84 (TQ 4/3) warp instructions per row
+// at 58% and 56% issue activity, against 97 and 95 at 53% for the CTA-wide 64-slot blocks
+// with a barrier each, clamps on every code and records assembled word by word: the 3 x
+// 20011-token rotated prompt's kernel 146 -> 107 us (2.6 TB/s), the 32K TQ prompt's
+// 82 -> 62 us.  What is left is the butterflies (14 packed adds per row), conversions,
+// radix groups and the exchange of stage 64.
 template <int BASE>
-__global__ void __launch_bounds__(kRows2Threads, rows2_ctas(BASE)) quantize_rows_kernel(QuantArgs a, int64_t n_hi, int64_t n_lo) {
-  extern __shared__ __align__(128) uint8_t rstage[];  // 2 stages of 256 half-row slots
-  __shared__ __align__(16) uint32_t smask[2][64];
-  const int tid = threadIdx.x;
-  const uint32_t nb_hi = (uint32_t)((n_hi + kRowSlots - 1) / kRowSlots);
-  const uint32_t per_bh = nb_hi + (uint32_t)((n_lo + kRowSlots - 1) / kRowSlots);
+__global__ void __launch_bounds__(kRowsThreads, kRowsCtas) quantize_rows_kernel(QuantArgs a, int64_t n_hi64, int64_t n_lo64) {
+  extern __shared__ __align__(128) uint8_t rstage[];  // per warp 2 stages of 32 half-row slots
+  __shared__ __align__(16) uint32_t smask_all[kRowsThreads / 32][64];
+  const int lane = threadIdx.x & 31;
+  // (the same in every lane: what follows from it stays in uniform registers)
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);
+  const int n_hi = (int)n_hi64, n_lo = (int)n_lo64;
+  const uint32_t u_hi = (uint32_t)(n_hi + kTileSlots - 1) / kTileSlots;
+  const uint32_t per_bh = u_hi + (uint32_t)(n_lo + kTileSlots - 1) / kTileSlots;
   const uint32_t total = (uint32_t)a.B * a.NL * a.H * per_bh;
-  auto tile = [&](uint32_t t) {
-    return rows_tile(t, nb_hi, per_bh, (uint32_t)n_hi, (uint32_t)n_lo, a.H, a.NL);
+  constexpr uint32_t kW = kRowsThreads / 32;
+  const uint32_t first = (uint32_t)((uint64_t)total * blockIdx.x / gridDim.x);
+  const uint32_t last = (uint32_t)((uint64_t)total * (blockIdx.x + 1) / gridDim.x);
+  const uint32_t begin = first + warp;
+  uint8_t* stages = rstage + warp * 2 * kWarpStageBytes;
+  uint32_t* smask = smask_all[warp];
+  const unsigned long long nz = opaque_neg_zero(smask);
+  // the thresholds of both pools, a zero one as +0 (tq_fields)
+  __shared__ float thr_sm[2][8];
+  if (BASE == SEMKV_BASE_TQ && threadIdx.x < 16) {
+    const int which = threadIdx.x >> 3, k = threadIdx.x & 7;
+    if (k < (which ? a.L_lo : a.L_hi) - 1)
+      thr_sm[which][k] = __fadd_rn((which ? a.thr_lo : a.thr_hi)[k], 0.0f);
+  }
+  __syncthreads();
+  pdl_wait();  // the slot maps and the rows come from earlier work on the stream
+  pdl_trigger();
+  auto advance = [&](RowsPos& p) {
+    p.r += kW;
+    while (p.r >= per_bh) {
+      p.r -= per_bh;
+      p.bhi++;
+    }
   };
-  // this thread's half row of block x into stage st (and, for tid < 64, a sign mask word)
-  auto issue = [&](const RowsTile& x, int st) {
-    if (tid < 64) {
-      const char2 s2 = *reinterpret_cast<const char2*>(a.signs + ((int64_t)x.l * a.H + x.h) * kHeadDim + 2 * tid);
-      smask[st][tid] = (s2.x < 0 ? 0x8000u : 0u) | (s2.y < 0 ? 0x80000000u : 0u);
-    }
-    const int i = tid >> 2;
-    if (i < x.nslots) {
-      const int64_t cap = x.hi ? a.hi_cap : a.lo_cap;
-      const int32_t* tokmap = (x.hi ? a.hi_tok : a.lo_tok) + (int64_t)x.b * cap + (x.hi ? a.hi_base : a.lo_base);
-      const int64_t tk = (int64_t)tokmap[x.s0 + i] - a.tok_base;
-      const int64_t bh = ((int64_t)x.b * a.NL + x.l) * a.H + x.h;
-      const uint16_t* src = (((tid >> 1) & 1) ? a.v : a.k) + (bh * a.Tsrc + tk) * kHeadDim + 64 * (tid & 1);
-      uint8_t* dst = rstage + st * kRows2StageBytes + tid * kHalfStride;
+  // this lane's token of the tile at p (a lane past the pool's slots takes the last one)
+  auto token = [&](const RowsPos& p) {
+    const uint32_t b = p.bhi / (uint32_t)(a.NL * a.H);
+    const bool hi = p.r < u_hi;
+    const int s = (int)(hi ? p.r : p.r - u_hi) * kTileSlots + (lane >> 2);
+    const int32_t* tokmap = hi ? a.hi_tok + (int64_t)b * a.hi_cap + a.hi_base
+                               : a.lo_tok + (int64_t)b * a.lo_cap + a.lo_base;
+    return tokmap[min(s, (hi ? n_hi : n_lo) - 1)];  // (tok_base comes off where it is used)
+  };
+  auto issue = [&](const RowsPos& p, int32_t tok, int st) {
+    const uint16_t* src = ((lane & 2) ? a.v : a.k) + ((int64_t)p.bhi * a.Tsrc + (tok - (int32_t)a.tok_base)) * kHeadDim + 64 * (lane & 1);
+    uint8_t* dst = stages + st * kWarpStageBytes + lane * kHalfStride;
 #pragma unroll
-      for (int c = 0; c < 8; ++c) cp_async16(dst + 16 * c, src + 8 * c);
-    }
+    for (int c = 0; c < 8; ++c) cp_async16(dst + 16 * c, src + 8 * c);
     cp_async_commit();
   };
-  uint32_t t = blockIdx.x;
-  RowsTile cur{};
-  if (t < total) {
-    cur = tile(t);
-    issue(cur, 0);
+  if (begin >= last) return;
+  const int trips = (int)((last - begin + kW - 1) / kW);
+  RowsPos cur;
+  cur.bhi = begin / per_bh;
+  cur.r = begin - cur.bhi * per_bh;
+  // the sign masks of (layer, head) lh
+  auto signs_of = [&](uint32_t lh, char2 (&s2)[2]) {
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+      s2[i] = *reinterpret_cast<const char2*>(a.signs + (int64_t)lh * kHeadDim + 2 * (lane + 32 * i));
+  };
+  auto put_masks = [&](const char2 (&s2)[2]) {
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+      smask[lane + 32 * i] = (s2[i].x < 0 ? 0x8000u : 0u) | (s2[i].y < 0 ? 0x80000000u : 0u);
+  };
+  uint32_t masked = cur.bhi % (uint32_t)(a.NL * a.H);  // whose masks are in smask
+  char2 s2[2];
+  int32_t tok = token(cur);
+  signs_of(masked, s2);
+  issue(cur, tok, 0);
+  RowsPos nxt = cur;
+  if (trips > 1) {
+    advance(nxt);
+    tok = token(nxt);
   }
-  for (int k = 0; t < total; t += gridDim.x, ++k) {
-    const int st = k & 1;
-    // this thread's copies of block k have landed; after the barrier every thread's have,
-    // and every warp is done with the other stage (block k - 1), which the copies of
-    // block k + 1 then take over
-    cp_async_wait<0>();
-    __syncthreads();
-    RowsTile nxt{};
-    if (t + gridDim.x < total) {
-      nxt = tile(t + gridDim.x);
-      issue(nxt, st ^ 1);
+  put_masks(s2);
+  for (int i = 0; i < trips; ++i) {
+    const int st = i & 1;
+    const uint32_t lh = cur.bhi % (uint32_t)(a.NL * a.H);
+    if (lh != masked) {
+      masked = lh;
+      signs_of(lh, s2);
+      __syncwarp();
+      put_masks(s2);
     }
-    uint8_t* stage = rstage + st * kRows2StageBytes;
-    switch (cur.hi ? a.L_hi : a.L_lo) {
+    cp_async_wait<0>();
+    __syncwarp();  // the tile has landed; the other stage's image has been stored
+    RowsPos after = nxt;
+    if (i + 1 < trips) {
+      issue(nxt, tok, st ^ 1);
+      if (i + 2 < trips) {
+        advance(after);
+        tok = token(after);
+      }
+    }
+    uint8_t* stage = stages + st * kWarpStageBytes;
+    const bool hi = cur.r < u_hi;
+    const int L = hi ? a.L_hi : a.L_lo;
+    const int s0 = (int)(hi ? cur.r : cur.r - u_hi) * kTileSlots;
+    const int ns = min(kTileSlots, (hi ? n_hi : n_lo) - s0);
+    uint8_t* rec = hi ? a.hi_pool + ((int64_t)cur.bhi * a.hi_cap + a.hi_base + s0) * record_bytes_rt(BASE, L)
+                      : a.lo_pool + ((int64_t)cur.bhi * a.lo_cap + a.lo_base + s0) * record_bytes_rt(BASE, L);
+    const float* thr = thr_sm[hi ? 0 : 1];
+    unsigned long long xp[32];
+    uint32_t param;
+    float invq, zq = 0.0f;
+    bool live;
+    rows_front<BASE>(L, stage, smask, nz, xp, param, invq, zq, live);
+    switch (L) {
 #define SEMKV_ROWS_CASE(LV) \
-      case LV: rows_half<BASE, LV>(a, cur.b, cur.l, cur.h, cur.hi, cur.s0, cur.nslots, stage, smask[st]); break;
+      case LV: rows_back<BASE, LV>(thr, stage, rec, ns, nz, xp, param, invq, zq, live); break;
       SEMKV_ROWS_CASE(2) SEMKV_ROWS_CASE(3) SEMKV_ROWS_CASE(4) SEMKV_ROWS_CASE(5)
       SEMKV_ROWS_CASE(6) SEMKV_ROWS_CASE(7) SEMKV_ROWS_CASE(8)
 #undef SEMKV_ROWS_CASE
       default: break;
     }
     cur = nxt;
+    nxt = after;
   }
 }
 // ------------------------------------------------- fake quantization ---------
@@ -1544,34 +1542,32 @@ cudaError_t launch_quantize_pack(const QuantArgs& a, int64_t n_hi, int num_sms,
     quantize_tq_dense_kernel<<<grid, kDenseThreads, kDenseSmem, stream>>>(a, n_hi, a.n - n_hi);
     return cudaGetLastError();
   }
-  // persistent CTAs (rows2_ctas per SM) over every block of both pools
+  // kRowsCtas CTAs per SM, each a range of the tiles of both pools
   const int64_t bhs = (int64_t)a.B * a.NL * a.H;
-  const int64_t blocks = bhs * ((n_hi + kRowSlots - 1) / kRowSlots +
-                                (a.n - n_hi + kRowSlots - 1) / kRowSlots);
-  int64_t ctas = (int64_t)(num_sms > 0 ? num_sms : 1) * rows2_ctas(a.base);
-  if (ctas > blocks) ctas = blocks;
+  const int64_t tiles = bhs * ((n_hi + kTileSlots - 1) / kTileSlots +
+                               (a.n - n_hi + kTileSlots - 1) / kTileSlots);
+  int64_t ctas = (int64_t)(num_sms > 0 ? num_sms : 1) * kRowsCtas;
+  constexpr int kRowWarps = kRowsThreads / 32;
+  if (ctas > (tiles + kRowWarps - 1) / kRowWarps) ctas = (tiles + kRowWarps - 1) / kRowWarps;
   if (ctas < 1) return cudaSuccess;
-  if (blocks + ctas > INT32_MAX) return cudaErrorInvalidValue;  // block indices are 32-bit
+  if (tiles > UINT32_MAX / 2) return cudaErrorInvalidValue;  // tile indices are 32-bit
   static bool rows_attr[kAttrDevices] = {};
   {
     const cudaError_t e = once_per_device(rows_attr, [] {
       cudaError_t r = cudaFuncSetAttribute(quantize_rows_kernel<SEMKV_BASE_AFFINE_HAD>,
                                            cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           2 * kRows2StageBytes);
+                                           kRowsThreads / 32 * 2 * kWarpStageBytes);
       if (r == cudaSuccess)
         r = cudaFuncSetAttribute(quantize_rows_kernel<SEMKV_BASE_TQ>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * kRows2StageBytes);
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, kRowsThreads / 32 * 2 * kWarpStageBytes);
       return r;
     });
     if (e != cudaSuccess) return e;
   }
-  if (a.base == SEMKV_BASE_AFFINE_HAD)
-    quantize_rows_kernel<SEMKV_BASE_AFFINE_HAD>
-        <<<(unsigned)ctas, kRows2Threads, 2 * kRows2StageBytes, stream>>>(a, n_hi, a.n - n_hi);
-  else
-    quantize_rows_kernel<SEMKV_BASE_TQ>
-        <<<(unsigned)ctas, kRows2Threads, 2 * kRows2StageBytes, stream>>>(a, n_hi, a.n - n_hi);
-  return cudaGetLastError();
+  return launch_pdl(a.base == SEMKV_BASE_AFFINE_HAD ? quantize_rows_kernel<SEMKV_BASE_AFFINE_HAD>
+                                                    : quantize_rows_kernel<SEMKV_BASE_TQ>,
+                    dim3((unsigned)ctas), dim3(kRowsThreads), kRowsThreads / 32 * 2 * kWarpStageBytes, stream, a,
+                    n_hi, a.n - n_hi);
 }
 
 }  // namespace semkv

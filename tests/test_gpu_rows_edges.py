@@ -1,0 +1,63 @@
+"""GPU edge sizes of the rows quantizer (TQ and rotated affine, 8-slot tiles, two lanes per
+row): pools of one slot to a few tiles, records that start off a 16-byte boundary (odd block
+appends), both pools and every level count, and rows whose parameters are limited or
+subnormal beside ordinary ones (the rows that still need their codes clamped).  Records are
+compared bit for bit with the oracle."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2608_28911_gb300 import synthetic
+from parity import Pair
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("base", [1, 2])
+@pytest.mark.parametrize("L_hi,L_lo,T,r,blk", [
+    (4, 3, 1, (0, 1), 1),       # one slot, then one at a time
+    (6, 5, 7, (1, 2), 3),
+    (8, 7, 9, (1, 3), 5),
+    (2, 4, 16, (1, 2), 7),
+    (5, 6, 33, (1, 1), 9),      # the high pool only, until blocks add low slots
+    (3, 8, 130, (26, 100), 31),
+])
+def test_rows_tiles_and_unaligned_appends_bit_exact(base, L_hi, L_lo, T, r, blk):
+    import torch
+    from paper_2608_28911_gb300 import semkv
+    n = 3 * blk
+    p = Pair(base, L_hi, L_lo, 2, 2, 3, 6, T, r[0], r[1], seed=900 + T, block=blk, extra_cap=n)
+    p.quantize()
+    p.assert_records_equal()
+    k, v = synthetic.kv(901 + T, 2, 2, 3, n)
+    s = synthetic.scores_zipf(902 + T, 2, n)
+    for i in range(3):
+        at = slice(i * blk, (i + 1) * blk)
+        p.stage(k[:, :, :, at], v[:, :, :, at], s[:, at])
+        semkv.semkv_append_block(p.desc, p.cache, 1, 2)
+        oracle.append_block(p.oc, 1, 2)
+    torch.cuda.synchronize()
+    p.assert_records_equal()
+    p.assert_untouched_past_counts()
+    assert int(p.cache.dev_error.item()) == 0
+
+
+@pytest.mark.parametrize("L", [2, 3, 4, 5, 6, 7, 8])
+def test_rotated_rows_with_limited_and_subnormal_parameters(L):
+    """Rows of one warp's tile that take the clamped codes beside rows that do not: values
+    near fp16's largest (offset and step limited), tiny values (subnormal steps, whose
+    rounding is coarse), constant and zero rows."""
+    import torch
+    from paper_2608_28911_gb300 import semkv
+    p = Pair(2, L, L, 1, 1, 2, 4, 40, 0, 1, seed=77)
+    rng = np.random.default_rng(5)
+    for x in (p.k, p.v):
+        x[0, 0, :, 3] = np.float16(60000.0) * np.sign(rng.standard_normal((2, 128)))
+        x[0, 0, :, 5] = np.float16(65504.0)
+        x[0, 0, :, 12] = (rng.integers(-3, 4, (2, 128)) * 2.0 ** -24).astype(np.float16)
+        x[0, 0, :, 13] = (rng.integers(-40, 41, (2, 128)) * 2.0 ** -24).astype(np.float16)
+        x[0, 0, :, 20] = 0.0
+        x[0, 0, :, 21] = np.float16(-2.5)
+    p.quantize()
+    torch.cuda.synchronize()
+    p.assert_records_equal()

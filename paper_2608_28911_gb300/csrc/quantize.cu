@@ -177,6 +177,8 @@ __device__ void affine_units(const QuantArgs& a, int b, int l, int h, bool hi, i
 
 // slot -> token maps of the tokens quantized by this call
 __global__ void scatter_tok_kernel(QuantArgs a) {
+  pdl_wait();  // the flags and slots come from earlier work on the stream
+  pdl_trigger();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= (int64_t)a.B * a.n) return;
   const int b = (int)(i / a.n), j = (int)(i % a.n);
@@ -1489,8 +1491,8 @@ cudaError_t launch_quantize_pack(const QuantArgs& a, int64_t n_hi, int num_sms,
   if (a.base == SEMKV_BASE_AFFINE) {
     if (!maps_ready) {
       const int64_t pairs = (int64_t)a.B * a.n;
-      scatter_tok_kernel<<<(unsigned)((pairs + 255) / 256), 256, 0, stream>>>(a);
-      const cudaError_t e = cudaGetLastError();
+      const cudaError_t e = launch_pdl(scatter_tok_kernel, dim3((unsigned)((pairs + 255) / 256)),
+                                       dim3(256), 0, stream, a);
       if (e != cudaSuccess) return e;
     }
     // grid x from a simple wave model: with R resident CTAs (kAffineCtas per SM), the pass takes
@@ -1520,8 +1522,8 @@ cudaError_t launch_quantize_pack(const QuantArgs& a, int64_t n_hi, int num_sms,
   // TQ, rotated affine and dense-rotation TQ: slot -> token maps, then the rows by slot
   if (!maps_ready) {
     const int64_t pairs = (int64_t)a.B * a.n;
-    scatter_tok_kernel<<<(unsigned)((pairs + 255) / 256), 256, 0, stream>>>(a);
-    const cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_pdl(scatter_tok_kernel, dim3((unsigned)((pairs + 255) / 256)),
+                                     dim3(256), 0, stream, a);
     if (e != cudaSuccess) return e;
   }
   if (a.base == SEMKV_BASE_TQ_DENSE) {

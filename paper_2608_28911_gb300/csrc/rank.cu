@@ -245,33 +245,45 @@ __global__ void __launch_bounds__(kThreads) rank_assign_kernel(RankArgs a) {
 // ---- long sequences on a thread-block cluster -----------------------------------
 // The same selection and sweep with one sequence spread over a cluster of kCluster
 // CTAs: CTA r keeps the keys of tokens [r chunk, (r+1) chunk) in its shared memory and
-// counts them into its own histograms; each pass every CTA sums the cluster's 256-bin
-// histograms through distributed shared memory and takes the same bin (the choice is
-// deterministic); for the sweep each CTA adds the (greater, equal) totals of the CTAs
-// before it, so every token sees the counts of all earlier tokens of the sequence.
+// counts them into histograms of its warps.  Per pass every CTA stores its 256 sums into
+// every CTA's shared memory (distributed shared memory; two buffers in turn, so that one
+// cluster barrier per pass orders both the stores and the reuse) and then selects the bin
+// from its own copy; the choice is the same everywhere.  From the same copy a CTA adds up
+// what the CTAs before it hold above the bin, and in it after the last pass: the
+// (greater, equal) counts that its sweep starts from, with no exchange of their own.
+//
+// Bound by latency: four passes of two CTA barriers and one cluster barrier.  32768 tokens:
+// 25.4 -> 12.4 us (131072: 35 -> 22) against reading the other CTAs' histograms bin by bin
+// behind two cluster barriers per pass, and two more for the totals.  The one-CTA kernel
+// stays below 8192 tokens (6000: 11.1 us on both; 4096: 9.3 against 10.7, and 16 sequences
+// of 4096 9.4 against 15).
 constexpr int kCluster = 8;
+__host__ __device__ inline uint32_t cluster_chunk(uint32_t T) { return (T + kCluster - 1) / kCluster; }
 
-__global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kThreads)
+template <int kCtas>  // CTAs per SM
+__global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kThreads, kCtas)
     rank_cluster_kernel(RankArgs a) {
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
   extern __shared__ uint32_t ckeys[];
-  __shared__ uint32_t hist[256];
-  __shared__ uint32_t whist[kThreads / 32][256];
-  __shared__ uint32_t sel_bin, sel_above;
+  __shared__ uint32_t whist[kThreads / 32][256];  // zero between passes
+  // sums of CTA r, bin 255 - i at [r][i] (descending keys)
+  __shared__ __align__(16) uint32_t tot[2][kCluster][256];
+  __shared__ uint32_t sel_bin, sel_k, gt_before, eq_before;
   __shared__ uint64_t warp_sums[32];
-  __shared__ uint64_t chunk_total;
   const int rank_in = (int)cluster.block_rank();
   const int b = blockIdx.x / kCluster;
   const float* s = a.scores + (int64_t)b * a.ld;
   uint8_t* is_high = a.is_high + (int64_t)b * a.T;
   uint32_t* slot = a.slot + (int64_t)b * a.T;
   const uint32_t T = (uint32_t)a.T;
-  const uint32_t chunk = (T + kCluster - 1) / kCluster;
+  const uint32_t chunk = cluster_chunk(T);
   const uint32_t c_begin = min(T, (uint32_t)rank_in * chunk);
   const uint32_t c_end = min(T, c_begin + chunk);
   const uint32_t nloc = c_end - c_begin;
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31;
+  pdl_wait();  // the scores come from earlier work on the stream
+  pdl_trigger();
 
   if (a.n_high == 0 || a.n_high == T) {  // the same branch in every CTA of the cluster
     const uint8_t all = a.n_high == T ? 1 : 0;
@@ -281,14 +293,17 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kThreads)
     }
     return;
   }
+  cluster.barrier_arrive();  // (waited for before the first store to another CTA)
   for (uint32_t i = tid; i < nloc; i += kThreads) ckeys[i] = order_key(s[c_begin + i]);
+  for (int i = tid; i < (kThreads / 32) * 256; i += kThreads) (&whist[0][0])[i] = 0;
+  if (tid == 0) gt_before = 0;
+  __syncthreads();
 
   uint32_t prefix = 0, mask = 0, k = a.n_high;
+#pragma unroll 1
   for (int pass = 0; pass < 4; ++pass) {
     const int shift = 24 - 8 * pass;
     uint32_t* wh = whist[tid >> 5];
-    for (int i = tid; i < (kThreads / 32) * 256; i += kThreads) (&whist[0][0])[i] = 0;
-    __syncthreads();
     for (uint32_t i0 = 0; i0 < nloc; i0 += kThreads * kSelItems) {
       uint32_t key[kSelItems];
 #pragma unroll
@@ -303,67 +318,75 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kThreads)
       }
     }
     __syncthreads();
-    for (int i = tid; i < 256; i += kThreads) {
-      uint32_t c = 0;
-#pragma unroll 8
-      for (int w = 0; w < kThreads / 32; ++w) c += whist[w][i];
-      hist[i] = c;
-    }
-    cluster.sync();  // every CTA's histogram is complete
-    if (tid < 32) {
-      // the cluster's counts, summed in CTA order (each CTA reaches the same totals)
-      uint32_t tot[8];
+    if (pass == 0) cluster.barrier_wait();  // every CTA of the cluster is running
+    if (tid < 256) {
+      uint32_t c[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
 #pragma unroll
-      for (int e = 0; e < 8; ++e) tot[e] = 0;
-      for (int r = 0; r < kCluster; ++r) {
-        const uint32_t* rh = cluster.map_shared_rank(hist, r);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) tot[e] += rh[255 - 8 * tid - e];
+      for (int w = 0; w < kThreads / 32; ++w) {
+        c[w & 7] += whist[w][tid];
+        whist[w][tid] = 0;
       }
-      // select_bin over the summed counts (lane l holds bins 255 - 8l .. 248 - 8l)
-      uint32_t sum = 0;
+      const uint32_t sum = ((c[0] + c[1]) + (c[2] + c[3])) + ((c[4] + c[5]) + (c[6] + c[7]));
+      uint32_t* mine = &tot[pass & 1][rank_in][255 - tid];
 #pragma unroll
-      for (int e = 0; e < 8; ++e) sum += tot[e];
+      for (int r = 0; r < kCluster; ++r) *cluster.map_shared_rank(mine, r) = sum;
+    }
+    cluster.sync();  // every CTA's sums are here (and the histograms are zero again)
+    if (tid < 32) {
+      // lane l holds bins 255 - 8l down to 248 - 8l: the cluster's counts, and those of
+      // the CTAs before this one
+      uint32_t c[8], bf[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) c[e] = bf[e] = 0;
+#pragma unroll
+      for (int r = 0; r < kCluster; ++r) {
+        const uint4* p = reinterpret_cast<const uint4*>(&tot[pass & 1][r][8 * lane]);
+        const uint4 x = p[0], y = p[1];
+        const uint32_t v[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          c[e] += v[e];
+          if (r < rank_in) bf[e] += v[e];
+        }
+      }
+      uint32_t sum = 0, before = 0;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        sum += c[e];
+        before += bf[e];
+      }
       uint32_t incl = sum;
 #pragma unroll
       for (int off = 1; off < 32; off <<= 1) {
         const uint32_t y = __shfl_up_sync(0xffffffffu, incl, off);
-        if (tid >= off) incl += y;
+        if (lane >= off) incl += y;
       }
       const uint32_t excl = incl - sum;
-      if (excl < k && incl >= k) {
+      const bool mine = excl < k && incl >= k;  // the bin is one of this lane's
+      uint32_t above = incl < k ? before : 0u;   // earlier CTAs' keys in bins above it
+      if (mine) {
         uint32_t cum = excl;
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
-          if (cum + tot[e] >= k) {
-            sel_bin = 255u - 8u * tid - (uint32_t)e;
-            sel_above = cum;
-            break;
+          if (cum < k && cum + c[e] >= k) {
+            sel_bin = 255u - 8u * lane - (uint32_t)e;
+            sel_k = k - cum;
+            eq_before = bf[e];
           }
-          cum += tot[e];
+          if (cum + c[e] < k) above += bf[e];
+          cum += c[e];
         }
       }
+      above = __reduce_add_sync(0xffffffffu, above);
+      if (lane == 0) gt_before += above;
     }
-    cluster.sync();  // every CTA has read the others' histograms: they may be reset
+    __syncthreads();
     prefix |= sel_bin << shift;
-    k -= sel_above;
+    k = sel_k;
     mask |= 0xFFu << shift;
   }
   const uint32_t theta = prefix, need = k;
-
-  // ---- this CTA's (greater, equal) totals, then the totals of the CTAs before it
-  {
-    uint64_t local = 0;
-    for (uint32_t i = tid; i < nloc; i += kThreads)
-      local += (ckeys[i] > theta ? 1ull : 0ull) | ((ckeys[i] == theta ? 1ull : 0ull) << 32);
-    uint64_t total;
-    (void)block_exclusive_scan(local, warp_sums, &total);
-    if (tid == 0) chunk_total = total;
-  }
-  cluster.sync();
-  uint64_t run = 0;
-  for (int r = 0; r < rank_in; ++r) run += *cluster.map_shared_rank(&chunk_total, r);
-  cluster.sync();  // no CTA leaves while another still reads its shared memory
+  uint64_t run = (uint64_t)gt_before | ((uint64_t)eq_before << 32);
 
   for (uint32_t c0 = 0; c0 < nloc; c0 += kThreads * kItems) {
     uint32_t keys[kItems];
@@ -497,18 +520,29 @@ size_t rank_workspace_words(int B, int T) { return (size_t)B * 4 * (size_t)T; }
 
 cudaError_t launch_rank_assign(const RankArgs& a, cudaStream_t stream) {
   if (a.B == 0 || a.T == 0) return cudaSuccess;
-  const uint32_t chunk = ((uint32_t)a.T + kCluster - 1) / kCluster;
+  const uint32_t chunk = cluster_chunk((uint32_t)a.T);
   if (a.T <= kThreads) {
     const cudaError_t e = launch_pdl(rank_small_kernel, dim3(a.B), dim3(kThreads), 0, stream, a);
     if (e != cudaSuccess) return e;
   } else if (a.T >= 8192 && chunk <= kSmemKeys) {
     static bool cattr_set[kAttrDevices] = {};
     const cudaError_t e = once_per_device(cattr_set, [] {
-      return cudaFuncSetAttribute(rank_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)(kSmemKeys * sizeof(uint32_t)));
+      cudaError_t r = cudaFuncSetAttribute(rank_cluster_kernel<1>,
+                                           cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)(kSmemKeys * sizeof(uint32_t)));
+      if (r == cudaSuccess)
+        r = cudaFuncSetAttribute(rank_cluster_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)(kSmemKeys * sizeof(uint32_t)));
+      return r;
     });
     if (e != cudaSuccess) return e;
-    rank_cluster_kernel<<<a.B * kCluster, kThreads, (size_t)chunk * sizeof(uint32_t), stream>>>(a);
+    // One CTA per SM (55 registers) while the clusters run together: a cluster lies inside
+    // one GPC, and 12 of them do (12 x 64K tokens: 15.6 us, 20.8 at two per SM and 32
+    // registers).  More sequences take two per SM (16 x 64K: 23.4 us, 29.5 in two waves).
+    const cudaError_t el =
+        launch_pdl(a.B <= 12 ? rank_cluster_kernel<1> : rank_cluster_kernel<2>,
+                   dim3(a.B * kCluster), dim3(kThreads), (size_t)chunk * sizeof(uint32_t), stream, a);
+    if (el != cudaSuccess) return el;
   } else {
     static bool attr_set[kAttrDevices] = {};
     const cudaError_t e = once_per_device(attr_set, [] {

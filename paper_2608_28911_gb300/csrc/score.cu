@@ -20,6 +20,8 @@ constexpr int kWarpsPerBlock = 8;
 __global__ void __launch_bounds__(kWarpsPerBlock * 32)
     score_kv_norm_kernel(ScoreArgs a) {
   const int lane = threadIdx.x & 31;
+  pdl_wait();  // the cache comes from earlier work on the stream
+  pdl_trigger();
   const int64_t total = (int64_t)a.B * a.T;
   const int64_t nw = (int64_t)gridDim.x * kWarpsPerBlock;
   for (int64_t w = (int64_t)blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5); w < total; w += nw) {
@@ -53,8 +55,7 @@ cudaError_t launch_score_kv_norm(const ScoreArgs& a, int num_sms, cudaStream_t s
   int64_t blocks = (total + kWarpsPerBlock - 1) / kWarpsPerBlock;
   const int64_t cap = (int64_t)num_sms * 32;  // grid-stride beyond this
   if (blocks > cap) blocks = cap;
-  score_kv_norm_kernel<<<(unsigned)blocks, kWarpsPerBlock * 32, 0, stream>>>(a);
-  return cudaGetLastError();
+  return launch_pdl(score_kv_norm_kernel, dim3((unsigned)blocks), dim3(kWarpsPerBlock * 32), 0, stream, a);
 }
 
 }  // namespace semkv

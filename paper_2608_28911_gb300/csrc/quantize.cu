@@ -235,16 +235,17 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kAffineCtas)
 constexpr int kRowSlots = 64;
 constexpr int kRowStride = 272;  // bytes per staged row: 256 + 16 spreads the banks
 constexpr int kTileSlots = 8;    // slots of a warp's tile
-constexpr int kRows2Threads = 256;
 constexpr int kHalfStride = 144;  // bytes per half-row slot: 128 + 16 (9 x 16 B: the 8 lanes
                                   // of a quarter warp reach distinct banks)
-constexpr int kRows2StageBytes = kRows2Threads * kHalfStride;
 constexpr int kWarpStageBytes = 32 * kHalfStride;
 // The quantizer: CTAs of 128 threads, 5 per SM (96 registers, 20 warps).  At 6 per SM (80
-// registers) the pairs spill and at 4 fewer warps hide the shuffles: the 3 x 20011 rotated
-// prompt took 159 us at 5, 166 at 24 warps, 182 at 16.
+// registers) the pairs spill and at 4 fewer warps hide the shuffles: the 32K TQ prompt takes
+// 87 us at 5, 103 at 6 and 92 at 4, the 3 x 20011 rotated one 133, 139 and 136.
 constexpr int kRowsThreads = 128;
 constexpr int kRowsCtas = 5;
+// Fake quantization: 4 per SM (128 registers; at 5 the two transforms spill, 144 against 128 us
+// for 4 layers x 16384 tokens of the rotated affine base, and at 3 fewer warps hide latency, 138).
+constexpr int kFakeCtas = 4;
 
 // packed binary32 pairs (two independent IEEE operations, rounded to nearest)
 __device__ __forceinline__ unsigned long long f2_add(unsigned long long a, unsigned long long b) {
@@ -325,6 +326,20 @@ __device__ __forceinline__ void fwht_half(unsigned long long (&xp)[32]) {
   for (int j = 0; j < 32; ++j) {
     const float lo = f2_lo(xp[j]), hi = f2_hi(xp[j]);
     xp[j] = f2_pack(__fadd_rn(lo, hi), __fsub_rn(lo, hi));
+  }
+}
+
+// Stage 64 across the two halves of a row (f: this lane's half, the partner is the lane
+// beside it).  Half 0 keeps a + b and half 1 a - b (a from half 0): fma(own, +-1, partner),
+// whose product is exact, rounds partner +- own once, which is that sum or difference.
+__device__ __forceinline__ void fwht_stage64(unsigned long long (&xp)[32], int f) {
+  const float sg = f ? -1.0f : 1.0f;
+  const unsigned long long sg2 = f2_pack(sg, sg);
+#pragma unroll
+  for (int j = 0; j < 32; ++j) {
+    const float plo = __shfl_xor_sync(0xffffffffu, f2_lo(xp[j]), 1);
+    const float phi = __shfl_xor_sync(0xffffffffu, f2_hi(xp[j]), 1);
+    xp[j] = f2_fma(xp[j], sg2, f2_pack(plo, phi));
   }
 }
 
@@ -481,20 +496,9 @@ __device__ __forceinline__ void rows_front(int L, const uint8_t* stage, const ui
     live = n != 0.0f;
     invq = live ? __fdiv_rn(1.0f, n) : 0.0f;
   }
-  // ---- butterflies: stages 1..32 in the thread, stage 64 with the partner half.  Half 0
-  // keeps a + b and half 1 a - b (a from half 0): fma(own, +-1, partner), whose product
-  // is exact, rounds partner +- own once, which is that sum or difference.
+  // ---- butterflies: stages 1..32 in the thread, stage 64 with the partner half
   fwht_half(xp);
-  {
-    const float sg = f ? -1.0f : 1.0f;
-    const unsigned long long sg2 = f2_pack(sg, sg);
-#pragma unroll
-    for (int j = 0; j < 32; ++j) {
-      const float plo = __shfl_xor_sync(0xffffffffu, f2_lo(xp[j]), 1);
-      const float phi = __shfl_xor_sync(0xffffffffu, f2_hi(xp[j]), 1);
-      xp[j] = f2_fma(xp[j], sg2, f2_pack(plo, phi));
-    }
-  }
+  fwht_stage64(xp, f);
   if constexpr (BASE == SEMKV_BASE_AFFINE_HAD) {
     float mn = INFINITY, mx = -INFINITY;
     const unsigned long long rs2 = f2_pack(kInvSqrtD, kInvSqrtD);
@@ -652,9 +656,8 @@ struct RowsPos {
   uint32_t bhi, r;
 };
 // Warps over tiles of 8 slots: a CTA takes a contiguous range, its warps the tiles in turn,
-// each warp with its own two-stage pipeline.  While a tile is quantized, the next one's half
-// rows (8 cp.async of 16 bytes per lane into the lane's slot) and the one after's token
-// indices are on their way.  No warp waits for another, and the positions stay in uniform
+// each warp with its own two-stage pipeline.  While a tile is quantized, the next one's
+// rows (8 cp.async of 16 bytes per lane) and the one after's token indices are on their way.  No warp waits for another, and the positions stay in uniform
 // registers (they leave room for the pairs, which otherwise spill).
 //
 // Bound by instruction issue: 76 (rotated affine) and 84 (TQ 4/3) warp instructions per row
@@ -707,11 +710,17 @@ __global__ void __launch_bounds__(kRowsThreads, kRowsCtas) quantize_rows_kernel(
                                : a.lo_tok + (int64_t)b * a.lo_cap + a.lo_base;
     return tokmap[min(s, (hi ? n_hi : n_lo) - 1)];  // (tok_base comes off where it is used)
   };
+  // row by row, so that an instruction reads 256 contiguous bytes of K and of V (slot i:
+  // chunk c of 16 bytes of row 2 i + kind goes to half 2 row + (c >> 3))
+  const int ch = lane & 15;
+  const uint16_t* kv = (lane < 16 ? a.k : a.v) + 8 * ch;
   auto issue = [&](const RowsPos& p, int32_t tok, int st) {
-    const uint16_t* src = ((lane & 2) ? a.v : a.k) + ((int64_t)p.bhi * a.Tsrc + (tok - (int32_t)a.tok_base)) * kHeadDim + 64 * (lane & 1);
-    uint8_t* dst = stages + st * kWarpStageBytes + lane * kHalfStride;
+    const uint16_t* src = kv + ((int64_t)p.bhi * a.Tsrc - a.tok_base) * kHeadDim;
+    uint8_t* dst = stages + st * kWarpStageBytes + (2 * (lane >> 4) + (ch >> 3)) * kHalfStride + (ch & 7) * 16;
 #pragma unroll
-    for (int c = 0; c < 8; ++c) cp_async16(dst + 16 * c, src + 8 * c);
+    for (int i = 0; i < kTileSlots; ++i)
+      cp_async16(dst + 4 * i * kHalfStride,
+                 src + (int64_t)__shfl_sync(0xffffffffu, tok, 4 * i) * kHeadDim);
     cp_async_commit();
   };
   if (begin >= last) return;
@@ -877,24 +886,10 @@ __global__ void __launch_bounds__(128, 5) fake_affine_kernel(FakeArgs a) {
   }
 }
 
-// Rotated affine and TQ: two threads per row, as the rows quantizer.  Persistent CTAs of
-// 256 threads over the 64-token blocks of every (sequence, layer, KV head): thread tid
-// holds half f = tid & 1 of row tid >> 1 (K of token tid >> 2 when bit 1 is 0, V when 1)
-// as 32 packed pairs (x_j, x_{j+32}), the next block's halves arriving by 16-byte
-// cp.async copies under the current block (one CTA barrier per block).  Both
-// transforms run the quantizer's butterflies (stages 1..32 in the thread, stage 64 with
-// the partner lane); the reconstruction is written back as fp16 with 16-byte stores.
-
-// stage 64 of the butterflies across the two halves of a row (half 0 keeps a + b, half 1
-// a - b, a from half 0): fma(own, +-1, partner) rounds partner +- own once
-__device__ __forceinline__ void fwht_stage64(unsigned long long (&xp)[32], unsigned long long sg2) {
-#pragma unroll
-  for (int j = 0; j < 32; ++j) {
-    const float plo = __shfl_xor_sync(0xffffffffu, f2_lo(xp[j]), 1);
-    const float phi = __shfl_xor_sync(0xffffffffu, f2_hi(xp[j]), 1);
-    xp[j] = f2_fma(xp[j], sg2, f2_pack(plo, phi));
-  }
-}
+// Rotated affine and TQ: the rows quantizer's tiles (8 tokens, two lanes per row, each warp
+// with its own two-stage pipeline) and its front half; then the values the codes stand for,
+// the same butterflies back, and the fp16 rows through the stage, so that both ways move
+// 512 contiguous bytes per instruction.
 
 // The codebook entry of each of a pair's two values: c = #{k : u > thr_k} over the
 // kLmax - 1 thresholds (the row's own L - 1 of them, then +inf), from the sign bits of
@@ -913,186 +908,188 @@ __device__ __forceinline__ unsigned long long tq_dequant2(unsigned long long u2,
   return f2_pack(cb[cl], cb[ch]);
 }
 
-// One half of a row (see above): slot holds its fp16 values, mask the sign masks of its
-// dims; out: the reconstruction's fp16 pairs for dims 64f + 2p, 64f + 2p + 1.
+// The values the row's codes stand for, in place of the rotated values in xp (pairs), and
+// the reconstruction's final factor: fp32(1/sqrt 128), or n / 128
 template <int BASE, int kLmax>
-__device__ __forceinline__ void fake_half(const uint8_t* slot, const uint32_t* mask, int f, int L,
-                                          bool sel_hi, const float (*cbs)[8], const FakeArgs& a,
-                                          uint32_t (&out)[32]) {
-  unsigned long long xp[32];
-  {
-    const uint4* src = reinterpret_cast<const uint4*>(slot);
-    const uint4* msk = reinterpret_cast<const uint4*>(mask);
-    uint32_t wv[32];
-#pragma unroll
-    for (int c = 0; c < 8; ++c) {
-      const uint4 u = src[c], m = msk[c];
-      wv[4 * c] = u.x ^ m.x; wv[4 * c + 1] = u.y ^ m.y;
-      wv[4 * c + 2] = u.z ^ m.z; wv[4 * c + 3] = u.w ^ m.w;
-    }
-#pragma unroll
-    for (int j = 0; j < 32; ++j) {
-      const uint32_t lo = wv[j >> 1], hi2 = wv[16 + (j >> 1)];
-      const int sh = 16 * (j & 1);
-      xp[j] = f2_pack(f16_to_f32((uint16_t)(lo >> sh)), f16_to_f32((uint16_t)(hi2 >> sh)));
-    }
-  }
-  const float sg = f ? -1.0f : 1.0f;
-  const unsigned long long sg2 = f2_pack(sg, sg);
-  float post;  // the reconstruction's final factor: fp32(1/sqrt 128), or n / 128
+__device__ __forceinline__ float fake_values(int L, unsigned long long nz, const float* thr,
+                                             const float* cb, bool active, uint32_t param,
+                                             float invq, float zq, bool live,
+                                             unsigned long long (&xp)[32]) {
+  const unsigned long long inv2 = f2_pack(invq, invq);
   if constexpr (BASE == SEMKV_BASE_AFFINE_HAD) {
-    // y = FWHT(z + s c);  x^_d = fp16((sign_d y_d) * fp32(1/sqrt 128))
-    fwht_half(xp);
-    fwht_stage64(xp, sg2);
-    float mn = INFINITY, mx = -INFINITY;
-#pragma unroll
-    for (int j = 0; j < 32; ++j) {
-      xp[j] = f2_pack(__fmul_rn(f2_lo(xp[j]), kInvSqrtD), __fmul_rn(f2_hi(xp[j]), kInvSqrtD));
-      mn = fminf(mn, fminf(f2_lo(xp[j]), f2_hi(xp[j])));
-      mx = fmaxf(mx, fmaxf(f2_lo(xp[j]), f2_hi(xp[j])));
-    }
-    mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, 1));
-    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-    if (mn == 0.0f) mn = 0.0f;
-    if (mx == 0.0f) mx = 0.0f;
-    uint16_t z16 = __half_as_ushort(__float2half_rd(mn));
-    if (z16 == 0xFC00u) z16 = 0xFBFFu;
-    const float z = f16_to_f32(z16);
-    const float sv = f16_to_f32(f16_param(__fdiv_rn(__fsub_rn(mx, z), (float)(L - 1))));
-    const float inv = sv > 0.0f ? __fdiv_rn(1.0f, sv) : 0.0f;
-    const unsigned long long z2 = f2_pack(z, z), inv2 = f2_pack(inv, inv), s2 = f2_pack(sv, sv);
+    const float sv = f16_to_f32((uint16_t)(param & 0xFFFFu)), top = (float)(L - 1);
+    const unsigned long long z2 = f2_pack(zq, zq), s2 = f2_pack(sv, sv);
     const unsigned long long mg2 = f2_pack(12582912.0f, 12582912.0f);
-    const float top = (float)(L - 1);
 #pragma unroll
-    for (int j = 0; j < 32; ++j) {
-      // c = rint(clamp((x - z) / s)) as an integer-valued float (every code 0 when s = 0);
-      // z + s c: s c is exact (an fp16 value times an integer below 8), so the fused
-      // multiply-add rounds as the separate multiply and add
-      const unsigned long long d = f2_mul(f2_sub(xp[j], z2), inv2);
-      const float ylo = fminf(fmaxf(f2_lo(d), 0.0f), top), yhi = fminf(fmaxf(f2_hi(d), 0.0f), top);
-      const unsigned long long c2 = f2_sub(f2_add(f2_pack(ylo, yhi), mg2), mg2);
-      xp[j] = f2_fma(s2, c2, z2);
+    for (int j = 0; j < 32; ++j) xp[j] = f2_mul_only(f2_sub(xp[j], z2), inv2, nz);
+    // (the clamp is needed only where the parameters were limited or subnormal: rows_back)
+    const bool plain = zq > -65504.0f && sv >= 0x1p-14f && sv < 65504.0f;
+    if (!__all_sync(0xffffffffu, plain || !active)) {
+#pragma unroll
+      for (int j = 0; j < 32; ++j)
+        xp[j] = f2_pack(fminf(fmaxf(f2_lo(xp[j]), 0.0f), top), fminf(fmaxf(f2_hi(xp[j]), 0.0f), top));
     }
-    post = kInvSqrtD;
+    // c = rint(...) as an integer-valued float (every code 0 when s = 0); z + s c: s c is
+    // exact (an fp16 value times an integer below 8), so the fused multiply-add rounds as
+    // the separate multiply and add
+#pragma unroll
+    for (int j = 0; j < 32; ++j) xp[j] = f2_fma(s2, f2_sub(f2_add(xp[j], mg2), mg2), z2);
+    return kInvSqrtD;
   } else {
-    // y = FWHT(cb[c]);  x^_d = fp16((sign_d y_d) * (n / 128))
-    float pn[8];
-#pragma unroll
-    for (int g = 0; g < 8; ++g) {
-      // (a square of an fp16 value is exact: a fused x * x + v rounds as the separate ops)
-      unsigned long long v = f2_mul(xp[4 * g], xp[4 * g]);
-#pragma unroll
-      for (int k = 1; k < 4; ++k) v = f2_add(v, f2_mul(xp[4 * g + k], xp[4 * g + k]));
-      const float plo = __shfl_xor_sync(0xffffffffu, f2_lo(v), 1);
-      const float phi = __shfl_xor_sync(0xffffffffu, f2_hi(v), 1);
-      const unsigned long long sp = f2_add(v, f2_pack(plo, phi));
-      pn[g] = __fadd_rn(f2_lo(sp), f2_hi(sp));
-    }
-#pragma unroll
-    for (int off = 4; off >= 1; off >>= 1)
-#pragma unroll
-      for (int g = 0; g < off; ++g) pn[g] = __fadd_rn(pn[g], pn[g + off]);
-    const float n = f16_to_f32(f16_param(__fsqrt_rn(pn[0])));
-    const float inv = n != 0.0f ? __fdiv_rn(1.0f, n) : 0.0f;
-    const float* tg = sel_hi ? a.thr_hi : a.thr_lo;
     unsigned long long t2[7];
 #pragma unroll
     for (int k = 0; k < kLmax - 1; ++k) {
       // a zero-norm row compares against +inf (all codes 0)
-      const float tk = (n != 0.0f && k < L - 1) ? __fadd_rn(__ldg(tg + k), 0.0f) : INFINITY;
+      const float tk = live && k < L - 1 ? thr[k] : INFINITY;
       t2[k] = f2_pack(tk, tk);
     }
-    fwht_half(xp);
-    fwht_stage64(xp, sg2);
-    const float* cb = cbs[sel_hi ? 0 : 1];
+    // u = y * fl(1/n), rounded before the comparisons subtract it
 #pragma unroll
-    for (int j = 0; j < 32; ++j) {
-      // u = y * fl(1/n), rounded before the comparisons subtract it
-      const unsigned long long u2 = f2_pack(__fmul_rn(f2_lo(xp[j]), inv), __fmul_rn(f2_hi(xp[j]), inv));
-      xp[j] = tq_dequant2<kLmax>(u2, t2, cb);
-    }
-    post = n * 0.0078125f;
-  }
-  fwht_half(xp);
-  fwht_stage64(xp, sg2);
-  // (sign_d y_d) * post = sign_d (y_d * post): the product rounds to fp16 next, no add
-  const unsigned long long p2 = f2_pack(post, post);
-#pragma unroll
-  for (int j = 0; j < 32; ++j) xp[j] = f2_mul(xp[j], p2);
-#pragma unroll
-  for (int p = 0; p < 16; ++p) {
-    const __half2 h0 = __floats2half2_rn(f2_lo(xp[2 * p]), f2_lo(xp[2 * p + 1]));
-    const __half2 h1 = __floats2half2_rn(f2_hi(xp[2 * p]), f2_hi(xp[2 * p + 1]));
-    out[p] = *reinterpret_cast<const uint32_t*>(&h0) ^ mask[p];
-    out[16 + p] = *reinterpret_cast<const uint32_t*>(&h1) ^ mask[16 + p];
+    for (int j = 0; j < 32; ++j)
+      xp[j] = tq_dequant2<kLmax>(f2_mul_only(xp[j], inv2, nz), t2, cb);
+    return f16_to_f32((uint16_t)param) * 0.0078125f;
   }
 }
 
+// Warps over tiles of 8 tokens of one (sequence, layer, head), the CTA's range in turn.
+// Bound by instruction issue: 4 layers x 16384 tokens of the rotated affine base 202 -> 128 us
+// (4.2 TB/s), TQ 4/3 249 -> 167, against 64-token blocks with a CTA barrier each, clamps on
+// every value and 16-byte stores a row apart.
 template <int BASE>
-__global__ void __launch_bounds__(kRows2Threads, 2) fake_rows_kernel(FakeArgs a, int Lmax) {
-  extern __shared__ __align__(128) uint8_t fstage[];  // 2 stages of 256 half-row slots
-  __shared__ __align__(16) uint32_t smask[2][64];
-  __shared__ float cbs[2][8];
-  const int tid = threadIdx.x, f = tid & 1, r = tid >> 1, i = r >> 1;
-  if (BASE == SEMKV_BASE_TQ && tid < 16) {
-    const int which = tid >> 3, k = tid & 7;
+__global__ void __launch_bounds__(kRowsThreads, kFakeCtas) fake_rows_kernel(FakeArgs a, int Lmax) {
+  extern __shared__ __align__(128) uint8_t fstage[];  // per warp 2 stages of 32 half-row slots
+  __shared__ __align__(16) uint32_t smask_all[kRowsThreads / 32][64];
+  __shared__ float cbs[2][8], thr_sm[2][8];
+  const int lane = threadIdx.x & 31, f = lane & 1;
+  // (the same in every lane: what follows from it stays in uniform registers)
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);
+  constexpr uint32_t kW = kRowsThreads / 32;
+  const uint32_t per_bh = (uint32_t)(a.T + kTileSlots - 1) / kTileSlots;
+  const uint32_t total = (uint32_t)a.B * a.NL * a.H * per_bh;
+  const uint32_t first = (uint32_t)((uint64_t)total * blockIdx.x / gridDim.x);
+  const uint32_t last = (uint32_t)((uint64_t)total * (blockIdx.x + 1) / gridDim.x);
+  const uint32_t begin = first + warp;
+  uint8_t* stages = fstage + warp * 2 * kWarpStageBytes;
+  uint32_t* smask = smask_all[warp];
+  const unsigned long long nz = opaque_neg_zero(smask);
+  if (BASE == SEMKV_BASE_TQ && threadIdx.x < 16) {
+    const int which = threadIdx.x >> 3, k = threadIdx.x & 7;
     const int L = which ? a.L_lo : a.L_hi;
     cbs[which][k] = k < L ? (which ? a.cent_lo : a.cent_hi)[k] : 0.0f;
+    // a zero threshold as +0 (tq_fields)
+    thr_sm[which][k] = k < L - 1 ? __fadd_rn((which ? a.thr_lo : a.thr_hi)[k], 0.0f) : INFINITY;
   }
-  const uint32_t nblk = (uint32_t)((a.T + kRowSlots - 1) / kRowSlots);
-  const uint32_t total = (uint32_t)a.B * a.NL * a.H * nblk;
-  // block t: (sequence, layer, head) index and first token
-  auto decode = [&](uint32_t t, uint32_t& bhi, int& t0) {
-    bhi = t / nblk;
-    t0 = (int)(t - bhi * nblk) * kRowSlots;
-  };
-  auto issue = [&](uint32_t t, int st) {
-    uint32_t bhi;
-    int t0;
-    decode(t, bhi, t0);
-    if (tid < 64) {
-      const uint32_t q = bhi / (uint32_t)a.H;
-      const int h = (int)(bhi - q * a.H), l = (int)(q % (uint32_t)a.NL);
-      const char2 s2 = *reinterpret_cast<const char2*>(a.signs + ((int64_t)l * a.H + h) * kHeadDim + 2 * tid);
-      smask[st][tid] = (s2.x < 0 ? 0x8000u : 0u) | (s2.y < 0 ? 0x80000000u : 0u);
+  __syncthreads();
+  if (begin >= last) return;
+  const int trips = (int)((last - begin + kW - 1) / kW);
+  auto advance = [&](RowsPos& p) {
+    p.r += kW;
+    while (p.r >= per_bh) {
+      p.r -= per_bh;
+      p.bhi++;
     }
-    if (i < a.T - t0) {
-      const uint16_t* src = ((r & 1) ? a.v : a.k) + ((int64_t)bhi * a.T + t0 + i) * kHeadDim + 64 * f;
-      uint8_t* dst = fstage + st * kRows2StageBytes + tid * kHalfStride;
+  };
+  // a tile's 8 K rows and 8 V rows are 2 KB each: chunk c of 16 bytes of row 2 t + kind goes
+  // to half 2 row + (c >> 3)
+  const int ch = lane & 15;
+  auto issue = [&](const RowsPos& p, int st) {
+    const int t0 = (int)p.r * kTileSlots, n = a.T - t0;
+    const int64_t row0 = (int64_t)p.bhi * a.T + t0;
+    uint8_t* dst = stages + st * kWarpStageBytes + (ch >> 3) * kHalfStride + (ch & 7) * 16;
 #pragma unroll
-      for (int c = 0; c < 8; ++c) cp_async16(dst + 16 * c, src + 8 * c);
+    for (int i = 0; i < 8; ++i) {
+      const int t = 2 * (i & 3) + (lane >> 4), kind = i >> 2;
+      if (t < n)
+        cp_async16(dst + (2 * t + kind) * 2 * kHalfStride,
+                   (kind ? a.v : a.k) + (row0 + t) * kHeadDim + 8 * ch);
     }
     cp_async_commit();
   };
-  uint32_t t = blockIdx.x;
-  if (t < total) issue(t, 0);
-  for (int k = 0; t < total; t += gridDim.x, ++k) {
-    const int st = k & 1;
+  // whether this lane's token of the tile is a high one
+  auto flag = [&](const RowsPos& p) -> uint32_t {
+    if (a.is_high == nullptr) return 1u;
+    const int64_t b = p.bhi / (uint32_t)(a.NL * a.H);
+    return a.is_high[b * a.T + min((int)p.r * kTileSlots + (lane >> 2), a.T - 1)];
+  };
+  RowsPos cur;
+  cur.bhi = begin / per_bh;
+  cur.r = begin - cur.bhi * per_bh;
+  issue(cur, 0);
+  uint32_t hi_cur = flag(cur), hi_nxt = 0;
+  uint32_t masked = 0xffffffffu;  // the (layer, head) whose masks are in smask
+  for (int i = 0; i < trips; ++i) {
+    const int st = i & 1;
+    const uint32_t lh = cur.bhi % (uint32_t)(a.NL * a.H);
+    if (lh != masked) {
+      masked = lh;
+      __syncwarp();
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const char2 s2 = *reinterpret_cast<const char2*>(a.signs + (int64_t)lh * kHeadDim + 2 * (lane + 32 * j));
+        smask[lane + 32 * j] = (s2.x < 0 ? 0x8000u : 0u) | (s2.y < 0 ? 0x80000000u : 0u);
+      }
+    }
     cp_async_wait<0>();
-    __syncthreads();  // the stage and its masks are published; the other stage is free
-    if (t + gridDim.x < total) issue(t + gridDim.x, st ^ 1);
-    uint32_t bhi;
-    int t0;
-    decode(t, bhi, t0);
-    const int b = (int)(bhi / ((uint32_t)a.H * a.NL));
-    const bool live = i < a.T - t0;
-    const bool sel_hi = a.is_high == nullptr || (live && a.is_high[(int64_t)b * a.T + t0 + i] != 0);
-    const int L = sel_hi ? a.L_hi : a.L_lo;
-    const uint8_t* slot = fstage + st * kRows2StageBytes + tid * kHalfStride;
-    uint32_t out[32];
+    __syncwarp();  // the tile has landed; the other stage's rows have been stored
+    RowsPos nxt = cur;
+    if (i + 1 < trips) {
+      advance(nxt);
+      issue(nxt, st ^ 1);
+      hi_nxt = flag(nxt);
+    }
+    uint8_t* stage = stages + st * kWarpStageBytes;
+    const int t0 = (int)cur.r * kTileSlots, n = a.T - t0;
+    const bool active = (lane >> 2) < n, hi = hi_cur != 0;
+    const int L = hi ? a.L_hi : a.L_lo;
+    unsigned long long xp[32];
+    uint32_t param;
+    float invq, zq = 0.0f, post = 0.0f;
+    bool live;
+    rows_front<BASE>(L, stage, smask, nz, xp, param, invq, zq, live);
     switch (BASE == SEMKV_BASE_TQ ? Lmax : 2) {
 #define SEMKV_FAKE_CASE(LV) \
-      case LV: fake_half<BASE, LV>(slot, smask[st] + 32 * f, f, L, sel_hi, cbs, a, out); break;
+      case LV: post = fake_values<BASE, LV>(L, nz, thr_sm[hi ? 0 : 1], cbs[hi ? 0 : 1], active, param, invq, zq, live, xp); break;
       SEMKV_FAKE_CASE(2) SEMKV_FAKE_CASE(3) SEMKV_FAKE_CASE(4) SEMKV_FAKE_CASE(5)
       SEMKV_FAKE_CASE(6) SEMKV_FAKE_CASE(7) SEMKV_FAKE_CASE(8)
 #undef SEMKV_FAKE_CASE
       default: break;
     }
-    if (live) {
-      uint4* dst = reinterpret_cast<uint4*>(((r & 1) ? a.v_out : a.k_out) + ((int64_t)bhi * a.T + t0 + i) * kHeadDim + 64 * f);
+    // ---- back: the butterflies, then sign_d (y_d * post) as fp16 into the lane's slot
+    fwht_half(xp);
+    fwht_stage64(xp, f);
+    {
+      const unsigned long long p2 = f2_pack(post, post);
+      uint32_t out[32];
 #pragma unroll
-      for (int c = 0; c < 8; ++c) dst[c] = make_uint4(out[4 * c], out[4 * c + 1], out[4 * c + 2], out[4 * c + 3]);
+      for (int p = 0; p < 16; ++p) {
+        const unsigned long long x = f2_mul(xp[2 * p], p2), y = f2_mul(xp[2 * p + 1], p2);
+        const __half2 h0 = __floats2half2_rn(f2_lo(x), f2_lo(y));
+        const __half2 h1 = __floats2half2_rn(f2_hi(x), f2_hi(y));
+        out[p] = *reinterpret_cast<const uint32_t*>(&h0);
+        out[16 + p] = *reinterpret_cast<const uint32_t*>(&h1);
+      }
+      const uint4* msk = reinterpret_cast<const uint4*>(smask + 32 * f);
+      uint4* slot = reinterpret_cast<uint4*>(stage + lane * kHalfStride);
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        const uint4 m = msk[c];
+        slot[c] = make_uint4(out[4 * c] ^ m.x, out[4 * c + 1] ^ m.y, out[4 * c + 2] ^ m.z, out[4 * c + 3] ^ m.w);
+      }
     }
+    __syncwarp();
+    {
+      const int64_t row0 = (int64_t)cur.bhi * a.T + t0;
+      const uint8_t* src = stage + (ch >> 3) * kHalfStride + (ch & 7) * 16;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const int t = 2 * (j & 3) + (lane >> 4), kind = j >> 2;
+        if (t < n)
+          reinterpret_cast<uint4*>((kind ? a.v_out : a.k_out) + (row0 + t) * kHeadDim)[ch] =
+              *reinterpret_cast<const uint4*>(src + (2 * t + kind) * 2 * kHalfStride);
+      }
+    }
+    cur = nxt;
+    hi_cur = hi_nxt;
   }
 }
 
@@ -1459,28 +1456,27 @@ cudaError_t launch_fake_quant(const FakeArgs& a, int num_sms, cudaStream_t strea
     return cudaGetLastError();
   }
   static bool attr_set[kAttrDevices] = {};
+  constexpr int kSmem = kRowsThreads / 32 * 2 * kWarpStageBytes;
   const cudaError_t e = once_per_device(attr_set, [] {
     cudaError_t r = cudaFuncSetAttribute(fake_rows_kernel<SEMKV_BASE_AFFINE_HAD>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         2 * kRows2StageBytes);
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
     if (r == cudaSuccess)
       r = cudaFuncSetAttribute(fake_rows_kernel<SEMKV_BASE_TQ>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * kRows2StageBytes);
+                               cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
     return r;
   });
   if (e != cudaSuccess) return e;
-  // persistent: 2 CTAs of 256 threads per SM (128 registers: both transforms' pairs and
-  // the dequantization constants spill at 80); block indices are 32-bit
-  if (bhs * nblk > INT32_MAX / 2) return cudaErrorInvalidValue;
-  int64_t ctas = (int64_t)(num_sms > 0 ? num_sms : 1) * 2;
-  if (ctas > bhs * nblk) ctas = bhs * nblk;
+  // tile indices are 32-bit (and a call of this size was refused by its 64-token blocks)
+  const int64_t tiles = bhs * (((int64_t)a.T + kTileSlots - 1) / kTileSlots);
+  if (bhs * nblk > INT32_MAX / 2 || tiles > UINT32_MAX / 2) return cudaErrorInvalidValue;
+  constexpr int kRowWarps = kRowsThreads / 32;
+  int64_t ctas = (int64_t)(num_sms > 0 ? num_sms : 1) * kFakeCtas;
+  if (ctas > (tiles + kRowWarps - 1) / kRowWarps) ctas = (tiles + kRowWarps - 1) / kRowWarps;
   const int Lmax = a.L_hi > a.L_lo ? a.L_hi : a.L_lo;
   if (a.base == SEMKV_BASE_AFFINE_HAD)
-    fake_rows_kernel<SEMKV_BASE_AFFINE_HAD>
-        <<<(unsigned)ctas, kRows2Threads, 2 * kRows2StageBytes, stream>>>(a, Lmax);
+    fake_rows_kernel<SEMKV_BASE_AFFINE_HAD><<<(unsigned)ctas, kRowsThreads, kSmem, stream>>>(a, Lmax);
   else
-    fake_rows_kernel<SEMKV_BASE_TQ>
-        <<<(unsigned)ctas, kRows2Threads, 2 * kRows2StageBytes, stream>>>(a, Lmax);
+    fake_rows_kernel<SEMKV_BASE_TQ><<<(unsigned)ctas, kRowsThreads, kSmem, stream>>>(a, Lmax);
   return cudaGetLastError();
 }
 

@@ -61,3 +61,37 @@ def test_rotated_rows_with_limited_and_subnormal_parameters(L):
     p.quantize()
     torch.cuda.synchronize()
     p.assert_records_equal()
+
+
+@pytest.mark.parametrize("base,L_hi,L_lo", [(1, 4, 3), (1, 2, 8), (2, 6, 5), (2, 3, 7)])
+@pytest.mark.parametrize("T,mixed", [(1, False), (7, True), (8, True), (9, True), (257, False)])
+def test_fake_rows_tile_edges_bit_exact(base, L_hi, L_lo, T, mixed):
+    """Fake quantization of the rotated bases at the edges of its 8-token tiles, with a row of
+    limited parameters, one of subnormal steps and a zero row."""
+    import torch
+    from paper_2608_28911_gb300 import semkv
+    B, NL, H = 2, 2, 3
+    k, v = synthetic.kv(300 + T, B, NL, H, T)
+    rng = np.random.default_rng(T)
+    k[0, 0, 1, T // 2] = np.float16(60000.0) * np.sign(rng.standard_normal(128)).astype(np.float16)
+    k[1, 1, 0, 0] = (rng.integers(-3, 4, 128) * 2.0 ** -24).astype(np.float16)
+    v[1, 0, 2, T - 1] = 0.0
+    ih = (rng.random((B, T)) < 0.4).astype(np.uint8) if mixed else None
+    sg = synthetic.signs(301 + T, NL, H)
+    kw = dict(signs=sg)
+    if base == 1:
+        kw["cb_hi"], kw["cb_lo"] = [oracle.lloyd_max_gaussian(L)[1:3] for L in (L_hi, L_lo)]
+    desc = semkv.QuantDesc(base, L_hi, L_lo, signs=sg)
+    kt, vt = torch.from_numpy(k).cuda(), torch.from_numpy(v).cuda()
+    n, pad, canary = kt.numel(), 64, 0x7BCD
+    big = [torch.full((n + 2 * pad,), canary, dtype=torch.int16, device="cuda") for _ in range(2)]
+    ko, vo = [x[pad:pad + n].view(torch.float16).view(kt.shape) for x in big]
+    semkv.semkv_fake_quant(desc, kt, vt, ko, vo, is_high=None if ih is None else torch.from_numpy(ih).cuda())
+    torch.cuda.synchronize()
+    for x in big:
+        g = x.cpu().numpy()
+        assert np.all(g[:pad] == canary) and np.all(g[pad + n:] == canary)
+    want = oracle.fake_quant(base, L_hi, L_lo, synthetic.f16_bits(k), synthetic.f16_bits(v),
+                             is_high=ih, **kw)
+    for got, w in zip((ko, vo), want):
+        assert np.array_equal(got.cpu().numpy().view(np.uint16), w)

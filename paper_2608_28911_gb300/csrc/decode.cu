@@ -251,6 +251,21 @@ __device__ __forceinline__ Window load_window(const uint8_t* rec, int pos) {
   r.q2 = __funnelshift_r(w2, w3, sh);
   return r;
 }
+// the window of a K quarter (2 words) or a V half quarter (1 word) of an L-level row: the
+// four-level ones start on a word and need only those words
+template <int L, int WORDS>
+__device__ __forceinline__ Window load_row_window(const uint8_t* rec, int pos) {
+  if constexpr (L == 4) {
+    const uint32_t* w = reinterpret_cast<const uint32_t*>(rec) + (pos >> 5);
+    Window r;
+    r.q0 = w[0];
+    r.q1 = WORDS > 1 ? w[1] : 0u;
+    r.q2 = 0u;
+    return r;
+  } else {
+    return load_window(rec, pos);
+  }
+}
 // bits [p, p+n) of a window (p, n compile-time after unrolling)
 __device__ __forceinline__ uint32_t wbits(const Window& w, int p, int n) {
   const uint32_t mask = (1u << n) - 1u;
@@ -366,6 +381,26 @@ __device__ __forceinline__ void l5_tail_pairs(uint32_t ut, uint32_t& X0, uint32_
   X1 = bytes_to_h2(P1);
 }
 
+// ---- four-level codes by byte lookups ------------------------------------------
+// A 2-bit code masked out of a word as a nibble (w & 0x3333.., (w >> 2) & 0x3333..) is a
+// byte permute's selector: one permute looks four codes up in the high bytes of fp16 0, 1,
+// 2, 3 (their low bytes are zero), and one more per register lays two of them out as fp16
+// values: 17 instructions for 16 codes, where extracting, converting and pairing them one
+// at a time took 64.
+constexpr uint32_t kL4Lut = 0x42403C00u;
+// X[0]: codes 0, 2, 4, 6 of the word, X[1]: 8, 10, 12, 14, X[2]: 1, 3, 5, 7, X[3]: 9, ..., 15
+__device__ __forceinline__ void l4_lookup(uint32_t w, uint32_t (&X)[4]) {
+  const uint32_t e = w & 0x33333333u, o = (w >> 2) & 0x33333333u;
+  X[0] = __byte_perm(kL4Lut, 0u, e);  // (a permute reads the low 16 bits of its selector)
+  X[1] = __byte_perm(kL4Lut, 0u, e >> 16);
+  X[2] = __byte_perm(kL4Lut, 0u, o);
+  X[3] = __byte_perm(kL4Lut, 0u, o >> 16);
+}
+// the code of a 16-code word in half `half` of K register i (0..7) of that word
+__host__ __device__ constexpr int l4_code(int i, int half) {
+  return ((i >> 1) & 1) * 8 + (i >> 2) + 2 * (2 * (i & 1) + half);
+}
+
 // F side of S = Q' F^T: the fp16 F-value pairs of one quarter row of one token (both
 // halves are the same token), as the B fragments of the 8 k-steps: slot p = 2j + i
 // goes to f[j][i].  Slot p < kHalf*G holds F_k of symbols s and s + kHalf (s = p / G,
@@ -385,6 +420,14 @@ __device__ __forceinline__ void k_quarter(const Window& w, uint32_t (&f)[8][2]) 
     uint32_t ft[2];
     D::tail(wbits(w, 70, 5), ft);
     h[15] = hsub1024(fpair(ft[0], ft[1]));
+  } else if constexpr (L == 4) {
+#pragma unroll
+    for (int wd = 0; wd < 2; ++wd) {
+      uint32_t X[4];
+      l4_lookup(wd ? w.q1 : w.q0, X);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) h[8 * wd + i] = __byte_perm(X[i >> 1], 0u, (i & 1) ? 0x3424 : 0x1404);
+    }
   } else {
 #pragma unroll
     for (int s = 0; s < D::kHalf; ++s) {
@@ -415,6 +458,7 @@ __device__ __forceinline__ float k_coef(const QT* qrow, int t, int p, int half) 
   using D = Dec<L>;
   using F = typename D::F;
   const int base = 32 * t;
+  if constexpr (L == 4) return qval(qrow, base + 16 * (p >> 3) + l4_code(p & 7, half));
   if (F::R > 0 && p == 15)
     return half == 0 ? qval(qrow, base + 30) - (float)L * qval(qrow, base + 31)
                      : qval(qrow, base + 31);
@@ -458,6 +502,18 @@ __device__ __forceinline__ void v_half_pair(const Window& wa, const Window& wb, 
     uint32_t X0, X1;
     l5_tail_pairs(fpair(wbits_rt(wa, tpos, 5), wbits_rt(wb, tpos, 5)), X0, X1);
     h[15] = hh ? hdigit<5>(X0, X1) : X0;
+  } else if constexpr (L == 4) {
+    // both tokens' words, then per two codes one permute pairs the tokens' bytes and two
+    // spread them to fp16
+    uint32_t Xa[4], Xb[4];
+    l4_lookup(wa.q0, Xa);
+    l4_lookup(wb.q0, Xb);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const uint32_t y = __byte_perm(Xa[i >> 1], Xb[i >> 1], (i & 1) ? 0x7362 : 0x5140);
+      h[l4_code(i, 0)] = __byte_perm(y, 0u, 0x1404);
+      h[l4_code(i, 1)] = __byte_perm(y, 0u, 0x3424);
+    }
   } else {
 #pragma unroll
     for (int j = 0; j < D::kHalf; ++j) {
@@ -568,16 +624,16 @@ __device__ void run_pool(const DecodeArgs& a, const Shared& sh, uint8_t* ring, u
   const float qscale =
       qmax > 0.0f ? pow2_floor(fminf(8192.0f / ((float)(L + 1) * qmax), 1e30f)) : 1.0f;
   // A fragments of the 8 k-steps, {hi 2j, lo 2j, hi 2j+1, lo 2j+1} per lane, the same
-  // for every warp of the CTA: warp 0 stores them in shared memory, every warp loads
+  // for every warp of the CTA: warp j stores step j in shared memory, every warp loads
   // its lane's fragment (one conflict-free 16-byte load per k-step)
+  static_assert(kWarps == 8, "one warp per coefficient step");
   uint4* aq = aq_all + lane;
   __syncthreads();  // the previous pool's fragments and the merge area are no longer read
-#pragma unroll
-  for (int j = 0; j < 8 && warp == 0; ++j) {
+  {
     uint32_t r[4];
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
-      const int p = 2 * j + i;
+      const int p = 2 * warp + i;
       float c0 = 0.0f, c1 = 0.0f;
       if (live && !upper) {
         if (CODEC == 0 && a.base != SEMKV_BASE_AFFINE_HAD) {
@@ -590,7 +646,7 @@ __device__ void run_pool(const DecodeArgs& a, const Shared& sh, uint8_t* ring, u
       }
       split_h2(c0, c1, r[2 * i], r[2 * i + 1]);
     }
-    aq[32 * j] = make_uint4(r[0], r[1], r[2], r[3]);
+    aq[32 * warp] = make_uint4(r[0], r[1], r[2], r[3]);
   }
   __syncthreads();  // every warp of the CTA runs this pool with the same level count
   const float cS = a.scale_log2 / qscale;   // logit weight of s_k * S
@@ -638,8 +694,8 @@ __device__ void run_pool(const DecodeArgs& a, const Shared& sh, uint8_t* ring, u
     float c0[4] = {0.f, 0.f, 0.f, 0.f}, c1[4] = {0.f, 0.f, 0.f, 0.f};
     {
       uint32_t f0[8][2], f1[8][2];
-      k_quarter<L>(load_window(tb + g * kRec, t * F::QB), f0);
-      k_quarter<L>(load_window(tb + (g + 8) * kRec, t * F::QB), f1);
+      k_quarter<L>(load_row_window<L, 2>(tb + g * kRec, t * F::QB), f0);
+      k_quarter<L>(load_row_window<L, 2>(tb + (g + 8) * kRec, t * F::QB), f1);
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
         const uint4 A = aq[32 * j];
@@ -773,10 +829,10 @@ __device__ void run_pool(const DecodeArgs& a, const Shared& sh, uint8_t* ring, u
     // ---- O^T += C^T P'^T
     {
       uint32_t VA[8][4];
-      v_half_pair<L, 0>(load_window(tb + (2 * t) * kRec, vpos),
-                        load_window(tb + (2 * t + 1) * kRec, vpos), tpos, hh, VA);
-      v_half_pair<L, 2>(load_window(tb + (2 * t + 8) * kRec, vpos),
-                        load_window(tb + (2 * t + 9) * kRec, vpos), tpos, hh, VA);
+      v_half_pair<L, 0>(load_row_window<L, 1>(tb + (2 * t) * kRec, vpos),
+                        load_row_window<L, 1>(tb + (2 * t + 1) * kRec, vpos), tpos, hh, VA);
+      v_half_pair<L, 2>(load_row_window<L, 1>(tb + (2 * t + 8) * kRec, vpos),
+                        load_row_window<L, 1>(tb + (2 * t + 9) * kRec, vpos), tpos, hh, VA);
 #pragma unroll
       for (int m = 0; m < 8; ++m) {
         mma16816(st.O[m], VA[m][0], VA[m][1], VA[m][2], VA[m][3], b0, b1);
@@ -1424,55 +1480,93 @@ __global__ void qrot_dense_kernel(DecodeArgs a) {
 
 // ------------------------------------------------------- fp16 stage tokens ----
 
-// Staged tokens are few (< block): one warp per token, lane = 4 dims, CUDA cores.
-// Writes rows in natural dim order and zs = 0.
-__device__ void run_stage(const DecodeArgs& a, const Shared& sh, int b, int h, int G,
-                          float* m_out, float* l_out, float* z_out, float* o_out) {
+// Staged tokens are few (at most a block): CUDA cores, in two passes with the logits between
+// them in shared memory, so that no token waits for the one before it.
+//  1. Logits: a warp takes four tokens at a time, 8 lanes per token with 16 dims each (three
+//     shuffles per head).  Then every warp takes the maximum per head.
+//  2. Weighted sums: a warp takes tokens warp, warp + 8, ...; lane = 4 dims.
+// Bound by latency: two rounds of loads instead of one round, a reduction over 32 lanes and
+// an exponential per token and head in a serial chain (STAGEFIG).
+// Writes rows in natural dim order and zs = 0.  logits: [G][stage_n rounded up to 32].
+constexpr int kStageRowBytes = (kWarps * 8 * kMoStride + 8 * 128) * 4;
+__host__ __device__ inline int stage_pad(int n) { return (n + 31) / 32 * 32; }
+
+struct MergeArea {
+  float m[kMaxWarps * 8], l[kMaxWarps * 8], z[kMaxWarps * 8];
+  float scale[kMaxWarps * 8], cta_z[8];
+};
+
+__device__ void run_stage(const DecodeArgs& a, Shared& sh, int b, int h, int G, MergeArea& mg,
+                          float* o_out, float* logits) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  float qf[8][4];
+  const int n = a.stage_n, pad = stage_pad(n);
+  const int64_t base = (((int64_t)b * a.NL + a.layer) * a.H + h) * a.block;
+  for (int i = threadIdx.x; i < G * 128; i += kThreads)
+    sh.qr[i >> 7][i & 127] = f16_to_f32(a.q[((int64_t)b * a.Hq + h * G) * 128 + i]);
+  __syncthreads();
+  {
+    // 8-byte pieces (the stage's alignment): lane e of a token takes pieces e, e + 8, ...
+    const int sub = lane >> 3, e = lane & 7;
+    for (int t0 = 4 * warp; t0 < n; t0 += 4 * kWarps) {
+      const int t = min(t0 + sub, n - 1);
+      const uint2* kr = reinterpret_cast<const uint2*>(a.stage_k + (base + t) * 128);
+      float x[16];
 #pragma unroll
-  for (int c = 0; c < 8; ++c)
+      for (int j = 0; j < 4; ++j) {
+        const uint2 u = kr[e + 8 * j];
+        x[4 * j] = f16_to_f32((uint16_t)(u.x & 0xFFFF));
+        x[4 * j + 1] = f16_to_f32((uint16_t)(u.x >> 16));
+        x[4 * j + 2] = f16_to_f32((uint16_t)(u.y & 0xFFFF));
+        x[4 * j + 3] = f16_to_f32((uint16_t)(u.y >> 16));
+      }
+      for (int c = 0; c < G; ++c) {
+        float d = 0.0f;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) qf[c][j] = c < G ? f16_to_f32(sh.q[c][4 * lane + j]) : 0.0f;
-  float m[8], l[8], o[8][4];
+        for (int j = 0; j < 4; ++j) {
+          const float4 q = *reinterpret_cast<const float4*>(&sh.qr[c][32 * j + 4 * e]);
+          d += q.x * x[4 * j] + q.y * x[4 * j + 1] + q.z * x[4 * j + 2] + q.w * x[4 * j + 3];
+        }
+#pragma unroll
+        for (int off = 4; off >= 1; off >>= 1) d += __shfl_xor_sync(0xffffffffu, d, off);
+        if (e == 0 && t0 + sub < n) logits[c * pad + t0 + sub] = d * a.scale_log2;
+      }
+    }
+  }
+  __syncthreads();
+  float M[8], l[8], o[8][4];
 #pragma unroll
   for (int c = 0; c < 8; ++c) {
-    m[c] = -INFINITY;
+    M[c] = -INFINITY;
     l[c] = 0.0f;
 #pragma unroll
     for (int j = 0; j < 4; ++j) o[c][j] = 0.0f;
+    if (c >= G) continue;
+    for (int t = lane; t < n; t += 32) M[c] = fmaxf(M[c], logits[c * pad + t]);
+#pragma unroll
+    for (int off = 16; off >= 1; off >>= 1) M[c] = fmaxf(M[c], __shfl_xor_sync(0xffffffffu, M[c], off));
   }
-  const int64_t base = (((int64_t)b * a.NL + a.layer) * a.H + h) * a.block;
-  for (int i = warp; i < a.stage_n; i += kWarps) {
-    const uint2 ku = *reinterpret_cast<const uint2*>(a.stage_k + (base + i) * 128 + 4 * lane);
-    const uint2 vu = *reinterpret_cast<const uint2*>(a.stage_v + (base + i) * 128 + 4 * lane);
-    const float kx[4] = {f16_to_f32(ku.x & 0xFFFF), f16_to_f32(ku.x >> 16),
-                         f16_to_f32(ku.y & 0xFFFF), f16_to_f32(ku.y >> 16)};
-    const float vx[4] = {f16_to_f32(vu.x & 0xFFFF), f16_to_f32(vu.x >> 16),
-                         f16_to_f32(vu.y & 0xFFFF), f16_to_f32(vu.y >> 16)};
+#pragma unroll 4
+  for (int t = warp; t < n; t += kWarps) {
+    const uint2 vu = *reinterpret_cast<const uint2*>(a.stage_v + (base + t) * 128 + 4 * lane);
+    const float vx[4] = {f16_to_f32((uint16_t)(vu.x & 0xFFFF)), f16_to_f32((uint16_t)(vu.x >> 16)),
+                         f16_to_f32((uint16_t)(vu.y & 0xFFFF)), f16_to_f32((uint16_t)(vu.y >> 16))};
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
       if (c >= G) break;
-      float d = qf[c][0] * kx[0] + qf[c][1] * kx[1] + qf[c][2] * kx[2] + qf[c][3] * kx[3];
+      const float p = exp2f(logits[c * pad + t] - M[c]);
+      l[c] += p;
 #pragma unroll
-      for (int off = 16; off >= 1; off >>= 1) d += __shfl_xor_sync(0xffffffffu, d, off);
-      const float lg = d * a.scale_log2;
-      const float mn = fmaxf(m[c], lg);
-      const float al = m[c] == -INFINITY ? 0.0f : exp2f(m[c] - mn);
-      const float pp = exp2f(lg - mn);
-      m[c] = mn;
-      l[c] = l[c] * al + pp;
-#pragma unroll
-      for (int j = 0; j < 4; ++j) o[c][j] = o[c][j] * al + pp * vx[j];
+      for (int j = 0; j < 4; ++j) o[c][j] += p * vx[j];
     }
   }
 #pragma unroll
   for (int c = 0; c < 8; ++c) {
     if (c >= G) break;
     if (lane == 0) {
-      m_out[warp * 8 + c] = m[c];
-      l_out[warp * 8 + c] = l[c];
-      z_out[warp * 8 + c] = 0.0f;
+      // a warp without tokens holds zeros at the common maximum
+      mg.m[warp * 8 + c] = M[c];
+      mg.l[warp * 8 + c] = l[c];
+      mg.z[warp * 8 + c] = 0.0f;
     }
 #pragma unroll
     for (int j = 0; j < 4; ++j) o_out[mo_at(warp * 8 + c, 4 * lane + j)] = o[c][j];
@@ -1498,10 +1592,24 @@ __host__ __device__ inline int pair_partials(const DecodePlan& P, int64_t bh) {
   return n_hi + n_lo + P.splits_st;
 }
 
-struct MergeArea {
-  float m[kMaxWarps * 8], l[kMaxWarps * 8], z[kMaxWarps * 8];
-  float scale[kMaxWarps * 8], cta_z[8];
-};
+// Walsh-Hadamard transform of 128 values over a warp (lane l holds dims 4l..4l+3): stages
+// 1, 2 inside the lane, then 4..64 across lanes, each (a + b, a - b) rounded to nearest
+__device__ __forceinline__ void wht_lanes(float (&w)[4], int lane) {
+  const float t0 = w[0] + w[1], t1 = w[0] - w[1], t2 = w[2] + w[3], t3 = w[2] - w[3];
+  w[0] = t0 + t2;
+  w[2] = t0 - t2;
+  w[1] = t1 + t3;
+  w[3] = t1 - t3;
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+    const bool upper = (lane >> k) & 1;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const float other = __shfl_xor_sync(0xffffffffu, w[j], 1 << k);
+      w[j] = upper ? other - w[j] : w[j] + other;
+    }
+  }
+}
 
 // the group's queries of pair (b, h) into shared memory, with their sums and maxima
 // (every thread of the CTA calls this; the caller orders it after earlier readers)
@@ -1558,20 +1666,7 @@ __device__ void load_group_q(const DecodeArgs& a, Shared& sh, int b, int h, int 
 #pragma unroll
     for (int j = 0; j < 4; ++j)
       w[j] = warp < G ? f16_to_f32(sh.q[warp][4 * lane + j]) * (float)sg[4 * lane + j] : 0.0f;
-    const float t0 = w[0] + w[1], t1 = w[0] - w[1], t2 = w[2] + w[3], t3 = w[2] - w[3];
-    w[0] = t0 + t2;
-    w[2] = t0 - t2;
-    w[1] = t1 + t3;
-    w[3] = t1 - t3;
-#pragma unroll
-    for (int k = 0; k < 5; ++k) {
-      const bool upper = (lane >> k) & 1;
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const float other = __shfl_xor_sync(0xffffffffu, w[j], 1 << k);
-        w[j] = upper ? other - w[j] : w[j] + other;
-      }
-    }
+    wht_lanes(w, lane);
     const float rs = a.base == SEMKV_BASE_AFFINE_HAD ? kInvSqrtD : 1.0f;
 #pragma unroll
     for (int j = 0; j < 4; ++j) sh.qr[warp][4 * lane + j] = w[j] * rs;
@@ -1603,7 +1698,8 @@ __device__ void load_group_q(const DecodeArgs& a, Shared& sh, int b, int h, int 
 // O columns are heads 2t, 2t+1 (for G <= 4, columns 4..7 hold the lo parts of heads
 // 0..3; they are written as rows 4..7 and folded in by merge_warps); rows 16m + g (+8)
 // are V rows u = 2m (+1) of lane group g, i.e. output dims v_dim(g, u).
-__device__ void affine_rows(WarpState& st, int L, int G, MergeArea& mg, float* merge_o) {
+template <int L>
+__device__ void affine_rows(WarpState& st, int G, MergeArea& mg, float* merge_o) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int g = lane >> 2, t = lane & 3;
   // reduce l and zs over the lanes that share a softmax head
@@ -1626,19 +1722,8 @@ __device__ void affine_rows(WarpState& st, int L, int G, MergeArea& mg, float* m
 #pragma unroll
       for (int m = 0; m < 8; ++m) {
 #pragma unroll
-        for (int r = 0; r < 2; ++r) {
-          int dim;
-          switch (L) {
-            case 2: dim = v_dim<2>(g, 2 * m + r); break;
-            case 3: dim = v_dim<3>(g, 2 * m + r); break;
-            case 4: dim = v_dim<4>(g, 2 * m + r); break;
-            case 5: dim = v_dim<5>(g, 2 * m + r); break;
-            case 6: dim = v_dim<6>(g, 2 * m + r); break;
-            case 7: dim = v_dim<7>(g, 2 * m + r); break;
-            default: dim = v_dim<8>(g, 2 * m + r); break;
-          }
-          merge_o[mo_at(warp * 8 + qh, dim)] = st.O[m][2 * r + c];
-        }
+        for (int r = 0; r < 2; ++r)
+          merge_o[mo_at(warp * 8 + qh, v_dim<L>(g, 2 * m + r))] = st.O[m][2 * r + c];
       }
     }
   }
@@ -1699,27 +1784,20 @@ __device__ void merge_warps(const DecodeArgs& a, int kind, int h, int G, MergeAr
     return;
   }
   __syncthreads();
-  if (rotated) {
-    // back from the rotated domain: o = S H o' (unnormalised transform, stages 1..64)
-    for (int hs = 1; hs < 128; hs <<= 1) {
-      for (int i = threadIdx.x; i < G * 64; i += NW * 32) {
-        const int qh = i >> 6, j = i & 63;
-        const int lo = (j / hs) * 2 * hs + (j % hs);
-        float* r = merged + qh * 128;
-        const float x = r[lo], y = r[lo + hs];
-        r[lo] = x + y;
-        r[lo + hs] = x - y;
-      }
-      __syncthreads();
-    }
-  }
-  const int8_t* sg = rotated ? a.signs + ((int64_t)a.layer * a.H + h) * 128 : nullptr;
-  // the rotated affine base stores rows in the orthonormal frame: x = S H u / sqrt(128)
+  // back from the rotated domain: o = S H o' (unnormalised transform, stages 1..64), one
+  // warp per head; the rotated affine base stores rows in the orthonormal frame: x = S H u /
+  // sqrt(128)
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int8_t* sg = a.signs + ((int64_t)a.layer * a.H + h) * 128;
   const float rs = a.base == SEMKV_BASE_AFFINE_HAD ? kInvSqrtD : 1.0f;
-  for (int i = threadIdx.x; i < G * 128; i += NW * 32) {
-    const int qh = i >> 7, d = i & 127;
-    const float o = merged[qh * 128 + d];
-    part[16 + qh * 128 + d] = rotated ? o * ((float)sg[d] * rs) : o;
+  if (warp < G) {
+    float x[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) x[j] = merged[warp * 128 + 4 * lane + j];
+    wht_lanes(x, lane);
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      part[16 + warp * 128 + 4 * lane + j] = x[j] * ((float)sg[4 * lane + j] * rs);
   }
   __syncthreads();  // the merge area (the ring) is free again
 }
@@ -1771,14 +1849,18 @@ __device__ void ring_fill_fast(uint8_t* ring, uint64_t* bars, const uint8_t* poo
   __syncwarp();
 }
 
-template <int L>
+template <int L, int CODEC = 0>
 __device__ void run_pool_any_g(const DecodeArgs& a, const Shared& sh, uint8_t* ring, uint4* aq_all,
                                uint64_t* bars, const uint8_t* pool_bh, int64_t count, int t0,
-                               int t1, int G, WarpState& st, int& ring_it) {
+                               int t1, int G, int& ring_it, MergeArea& mg, float* merge_o,
+                               int which = 0) {
+  WarpState st;
+  state_init(st);
   if (G <= 4)
-    run_pool<L, true>(a, sh, ring, aq_all, bars, pool_bh, count, t0, t1, G, st, ring_it, 0, true);
+    run_pool<L, true, CODEC>(a, sh, ring, aq_all, bars, pool_bh, count, t0, t1, G, st, ring_it, which, true);
   else
-    run_pool<L, false>(a, sh, ring, aq_all, bars, pool_bh, count, t0, t1, G, st, ring_it, 0, true);
+    run_pool<L, false, CODEC>(a, sh, ring, aq_all, bars, pool_bh, count, t0, t1, G, st, ring_it, which, true);
+  affine_rows<L>(st, G, mg, merge_o);
 }
 
 // Affine pools, balanced plan: CTA c takes the weighted range [c per, (c+1) per) of the
@@ -1832,19 +1914,14 @@ __global__ void __launch_bounds__(kThreads, kCtasAffine) decode_affine_kernel(De
         load_group_q(a, sh, b, h, G);
         loaded = bh;
       }
-      WarpState st;
-      state_init(st);
       switch (L) {
-        case 2: run_pool_any_g<2>(a, sh, ring, aq_all, bars, pool_bh, count, t0, t1, G, st, ring_it); break;
-        case 3: run_pool_any_g<3>(a, sh, ring, aq_all, bars, pool_bh, count, t0, t1, G, st, ring_it); break;
-        case 4: run_pool_any_g<4>(a, sh, ring, aq_all, bars, pool_bh, count, t0, t1, G, st, ring_it); break;
-        case 5: run_pool_any_g<5>(a, sh, ring, aq_all, bars, pool_bh, count, t0, t1, G, st, ring_it); break;
-        case 6: run_pool_any_g<6>(a, sh, ring, aq_all, bars, pool_bh, count, t0, t1, G, st, ring_it); break;
-        case 7: run_pool_any_g<7>(a, sh, ring, aq_all, bars, pool_bh, count, t0, t1, G, st, ring_it); break;
-        case 8: run_pool_any_g<8>(a, sh, ring, aq_all, bars, pool_bh, count, t0, t1, G, st, ring_it); break;
+#define SEMKV_POOL_CASE(LV) \
+        case LV: run_pool_any_g<LV>(a, sh, ring, aq_all, bars, pool_bh, count, t0, t1, G, ring_it, mg, merge_o); break;
+        SEMKV_POOL_CASE(2) SEMKV_POOL_CASE(3) SEMKV_POOL_CASE(4) SEMKV_POOL_CASE(5)
+        SEMKV_POOL_CASE(6) SEMKV_POOL_CASE(7) SEMKV_POOL_CASE(8)
+#undef SEMKV_POOL_CASE
         default: break;
       }
-      affine_rows(st, L, G, mg, merge_o);
       merge_warps(a, a.base == SEMKV_BASE_AFFINE_HAD ? 3 : 0, h, G, mg, merge_o,
                   a.partials + (bh * P.stride + slot) * kPartialFloats);
     }
@@ -1967,9 +2044,90 @@ __global__ void __launch_bounds__(NW * 32, NW == kWarps ? kCtasFast : 1)
   }
 }
 
-// TQ pools (KIND 1, one CTA per split) and the fp16 stage (KIND 2, one CTA per pair).
-template <int KIND>
-__global__ void __launch_bounds__(kThreads, kCtasOther) decode_kernel(DecodeArgs a) {
+// TQ pools, one CTA per split of one pool of a pair.
+__global__ void __launch_bounds__(kThreads, kCtasOther) decode_tq_kernel(DecodeArgs a) {
+  extern __shared__ __align__(128) uint8_t dyn[];
+  __shared__ Shared sh;
+  __shared__ MergeArea mg;
+  uint8_t* ring = dyn;
+  uint4* aq_all = reinterpret_cast<uint4*>(dyn + kRingBytes);
+  float* merge_o = reinterpret_cast<float*>(dyn);  // [kWarps][8][128] rows, then [8][128]
+  uint64_t* bars = &sh.bar[0][0];
+  const DecodePlan& P = a.plan;
+  const int b = blockIdx.z, h = blockIdx.y, split = blockIdx.x;
+  const int64_t bh = (int64_t)b * a.H + h;
+  const int G = a.Hq / a.H;
+  const int src = split < P.splits_hi ? 0 : 1;
+  const int s_idx = src == 0 ? split : split - P.splits_hi;
+  const int nsrc = src == 0 ? P.splits_hi : P.splits_lo;
+  const int ntiles = src == 0 ? P.tiles_hi : P.tiles_lo;
+  const int per = (ntiles + nsrc - 1) / nsrc;
+  const int t_begin = min(ntiles, s_idx * per), t_end = min(ntiles, t_begin + per);
+  const int L = src == 0 ? a.L_hi : a.L_lo;
+  const int64_t cap = src == 0 ? a.hi_cap : a.lo_cap;
+  const int64_t count = src == 0 ? a.hi_count : a.lo_count;
+  const uint8_t* pool = src == 0 ? a.hi_pool : a.lo_pool;
+  const int rec = record_bytes_rt(SEMKV_BASE_TQ, L);
+  const uint8_t* pool_bh = pool + (((int64_t)b * a.NL + a.layer) * a.H + h) * cap * rec;
+  if (threadIdx.x < kWarps * kStages) mbar_init(bars + threadIdx.x);
+  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  if (threadIdx.x < 16) {
+    const int which = threadIdx.x >> 3, k = threadIdx.x & 7;
+    sh.cb[which][k] = k < (which == 0 ? a.L_hi : a.L_lo) ? (which == 0 ? a.cb_hi : a.cb_lo)[k] : 0.0f;
+  }
+  __syncthreads();
+  pdl_wait();  // the records and queries (and the dense rotation's q') come from earlier work
+  pdl_trigger();
+  // centroids as cz + cs c (two levels; three when equally spaced), or for four exactly
+  // symmetric levels alpha phi + beta phi^3, phi = 2c - 3
+  const float* cb = sh.cb[src];
+  int path = 0;
+  if (L == 2 || (L == 3 && cb[1] - cb[0] == cb[2] - cb[1])) path = 1;
+  else if (L == 4 && cb[0] == -cb[3] && cb[1] == -cb[2]) path = 2;
+  if (threadIdx.x == 0) {
+    float cs = 0.0f, cz = 0.0f, c3 = 0.0f;
+    if (path == 1) {
+      cs = cb[1] - cb[0];
+      cz = cb[0];
+    } else if (path == 2) {
+      const float beta = (cb[3] - 3.0f * cb[2]) / 24.0f;
+      const float alpha = cb[2] - beta;
+      cs = 2.0f * alpha;
+      cz = -3.0f * alpha;
+      c3 = beta;
+    }
+    sh.cdec[src][0] = cs;
+    sh.cdec[src][1] = cz;
+    sh.cdec[src][2] = c3;
+  }
+  // the first copies run under the queries' loads and the coefficient fragments
+  int ring_it = 0;
+  if (path) ring_fill(ring, bars, pool_bh, (uint32_t)(kTile * rec), t_begin, t_end, ring_it);
+  load_group_q(a, sh, b, h, G);
+  int kind = 3;
+  if (path) {
+    if (L == 2)
+      run_pool_any_g<2, 1>(a, sh, ring, aq_all, bars, pool_bh, count, t_begin, t_end, G, ring_it, mg, merge_o, src);
+    else if (L == 3)
+      run_pool_any_g<3, 1>(a, sh, ring, aq_all, bars, pool_bh, count, t_begin, t_end, G, ring_it, mg, merge_o, src);
+    else
+      run_pool_any_g<4, 2>(a, sh, ring, aq_all, bars, pool_bh, count, t_begin, t_end, G, ring_it, mg, merge_o, src);
+  } else {
+    kind = 1;
+    switch (L) {
+#define SEMKV_TQ_CASE(LV) \
+      case LV: run_pool_tq<LV>(a, sh, src, pool_bh, count, t_begin, t_end, G, mg.m, mg.l, mg.z, merge_o); break;
+      SEMKV_TQ_CASE(2) SEMKV_TQ_CASE(3) SEMKV_TQ_CASE(4) SEMKV_TQ_CASE(5)
+      SEMKV_TQ_CASE(6) SEMKV_TQ_CASE(7) SEMKV_TQ_CASE(8)
+#undef SEMKV_TQ_CASE
+      default: break;
+    }
+  }
+  merge_warps(a, kind, h, G, mg, merge_o, a.partials + (bh * P.stride + split) * kPartialFloats);
+}
+
+// The fp16 stage, one CTA per pair.
+__global__ void __launch_bounds__(kThreads, kCtasOther) decode_stage_kernel(DecodeArgs a) {
   extern __shared__ __align__(128) uint8_t dyn[];
   __shared__ Shared sh;
   __shared__ MergeArea mg;
@@ -1978,129 +2136,18 @@ __global__ void __launch_bounds__(kThreads, kCtasOther) decode_kernel(DecodeArgs
   const int b = blockIdx.z, h = blockIdx.y;
   const int64_t bh = (int64_t)b * a.H + h;
   const int G = a.Hq / a.H;
-  int split = blockIdx.x;
-  if (KIND == 1) {
-    pdl_wait();  // the records and queries (and the dense rotation's q') come from earlier work
-    pdl_trigger();
+  if (!a.stage_overlaps_pools) pdl_wait();
+  int split = P.splits_hi + P.splits_lo;
+  if (P.balanced) {
+    int n_hi, n_lo;
+    pair_slots(P, bh, n_hi, n_lo);
+    split = n_hi + n_lo;
   }
-  if (KIND == 2 && !a.stage_overlaps_pools) pdl_wait();
-  if (KIND == 2) {
-    if (P.balanced) {
-      int n_hi, n_lo;
-      pair_slots(P, bh, n_hi, n_lo);
-      split = n_hi + n_lo;
-    } else {
-      split = P.splits_hi + P.splits_lo;
-    }
-  }
-  load_group_q(a, sh, b, h, G);
-  __shared__ int tq_path;  // TQ: 1 when this pool's codebook takes the tensor-core path
-  if (KIND == 1) {
-    if (threadIdx.x < 16) {
-      const int which = threadIdx.x >> 3, k = threadIdx.x & 7;
-      const int L = which == 0 ? a.L_hi : a.L_lo;
-      sh.cb[which][k] = k < L ? (which == 0 ? a.cb_hi : a.cb_lo)[k] : 0.0f;
-    }
-  }
-  __syncthreads();
-  if (KIND == 1) {
-    // rotated queries: sums and maxima for the tensor-core path
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    float s = 0.0f, mx = 0.0f;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const float x = sh.qr[warp][4 * lane + j];
-      s += x;
-      mx = fmaxf(mx, fabsf(x));
-    }
-#pragma unroll
-    for (int off = 16; off >= 1; off >>= 1) {
-      s += __shfl_xor_sync(0xffffffffu, s, off);
-      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-    }
-    if (lane == 0) {
-      sh.sumq[warp] = s;
-      sh.qmax[warp] = mx;
-    }
-    if (threadIdx.x == 0) {
-      // centroids as cz + cs c (two levels; three when equally spaced), or for four
-      // exactly symmetric levels alpha phi + beta phi^3, phi = 2c - 3
-      const int src0 = split < P.splits_hi ? 0 : 1;
-      const int L = src0 == 0 ? a.L_hi : a.L_lo;
-      const float* cb = sh.cb[src0];
-      int path = 0;
-      float cs = 0.0f, cz = 0.0f, c3 = 0.0f;
-      if (L == 2 || (L == 3 && cb[1] - cb[0] == cb[2] - cb[1])) {
-        path = 1;
-        cs = cb[1] - cb[0];
-        cz = cb[0];
-      } else if (L == 4 && cb[0] == -cb[3] && cb[1] == -cb[2]) {
-        path = 2;
-        const float beta = (cb[3] - 3.0f * cb[2]) / 24.0f;
-        const float alpha = cb[2] - beta;
-        cs = 2.0f * alpha;
-        cz = -3.0f * alpha;
-        c3 = beta;
-      }
-      sh.cdec[src0][0] = cs;
-      sh.cdec[src0][1] = cz;
-      sh.cdec[src0][2] = c3;
-      tq_path = path;
-    }
-  }
-  __syncthreads();
-  int kind = KIND;
-  if constexpr (KIND == 2) {
-    run_stage(a, sh, b, h, G, mg.m, mg.l, mg.z, merge_o);
-  } else {
-    const int src = split < P.splits_hi ? 0 : 1;
-    const int s_idx = src == 0 ? split : split - P.splits_hi;
-    const int nsrc = src == 0 ? P.splits_hi : P.splits_lo;
-    const int ntiles = src == 0 ? P.tiles_hi : P.tiles_lo;
-    const int per = (ntiles + nsrc - 1) / nsrc;
-    const int t_begin = min(ntiles, s_idx * per), t_end = min(ntiles, t_begin + per);
-    const int L = src == 0 ? a.L_hi : a.L_lo;
-    const int64_t cap = src == 0 ? a.hi_cap : a.lo_cap;
-    const int64_t count = src == 0 ? a.hi_count : a.lo_count;
-    const uint8_t* pool = src == 0 ? a.hi_pool : a.lo_pool;
-    const int rec = record_bytes_rt(SEMKV_BASE_TQ, L);
-    const uint8_t* pool_bh = pool + (((int64_t)b * a.NL + a.layer) * a.H + h) * cap * rec;
-    if (tq_path) {
-      uint8_t* ring = dyn;
-      uint4* aq_all = reinterpret_cast<uint4*>(dyn + kRingBytes);
-      uint64_t* bars = &sh.bar[0][0];
-      if (threadIdx.x < kWarps * kStages) mbar_init(bars + threadIdx.x);
-      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-      WarpState st;
-      state_init(st);
-      int ring_it = 0;
-      if (L == 2) {
-        if (G <= 4) run_pool<2, true, 1>(a, sh, ring, aq_all, bars, pool_bh, count, t_begin, t_end, G, st, ring_it, src);
-        else run_pool<2, false, 1>(a, sh, ring, aq_all, bars, pool_bh, count, t_begin, t_end, G, st, ring_it, src);
-      } else if (L == 3) {
-        if (G <= 4) run_pool<3, true, 1>(a, sh, ring, aq_all, bars, pool_bh, count, t_begin, t_end, G, st, ring_it, src);
-        else run_pool<3, false, 1>(a, sh, ring, aq_all, bars, pool_bh, count, t_begin, t_end, G, st, ring_it, src);
-      } else {
-        if (G <= 4) run_pool<4, true, 2>(a, sh, ring, aq_all, bars, pool_bh, count, t_begin, t_end, G, st, ring_it, src);
-        else run_pool<4, false, 2>(a, sh, ring, aq_all, bars, pool_bh, count, t_begin, t_end, G, st, ring_it, src);
-      }
-      affine_rows(st, L, G, mg, merge_o);
-      kind = 3;
-    } else {
-      switch (L) {
-#define SEMKV_TQ_CASE(LV) \
-        case LV: run_pool_tq<LV>(a, sh, src, pool_bh, count, t_begin, t_end, G, mg.m, mg.l, mg.z, merge_o); break;
-        SEMKV_TQ_CASE(2) SEMKV_TQ_CASE(3) SEMKV_TQ_CASE(4) SEMKV_TQ_CASE(5)
-        SEMKV_TQ_CASE(6) SEMKV_TQ_CASE(7) SEMKV_TQ_CASE(8)
-#undef SEMKV_TQ_CASE
-        default: break;
-      }
-    }
-  }
-  merge_warps(a, kind, h, G, mg, merge_o, a.partials + (bh * P.stride + split) * kPartialFloats);
+  run_stage(a, sh, b, h, G, mg, merge_o, reinterpret_cast<float*>(dyn + kStageRowBytes));
+  merge_warps(a, 2, h, G, mg, merge_o, a.partials + (bh * P.stride + split) * kPartialFloats);
   // a stage kernel that ran alongside the pool kernel completes only after it: the
   // combine, which waits for this kernel, then sees every pool partial too
-  if (KIND == 2) pdl_wait();
+  pdl_wait();
 }
 
 // merge the partials of each (b, qh): one warp per head, 4 dims per lane.  The lanes
@@ -2467,11 +2514,11 @@ cudaError_t launch_decode_attention(const DecodeArgs& a, cudaStream_t stream) {
                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  fast_ring_bytes<kFastWarps>() + kQbBytes);
       if (r == cudaSuccess)
-        r = cudaFuncSetAttribute(decode_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        r = cudaFuncSetAttribute(decode_tq_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  kRingBytes + kAqBytes);
       if (r == cudaSuccess)
-        r = cudaFuncSetAttribute(decode_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 kRingBytes);
+        r = cudaFuncSetAttribute(decode_stage_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 kStageRowBytes + 8 * stage_pad(1024) * 4);
       return r;
     });
     if (e != cudaSuccess) return e;
@@ -2488,7 +2535,7 @@ cudaError_t launch_decode_attention(const DecodeArgs& a, cudaStream_t stream) {
     }
     const int pool_splits = P.splits_hi + P.splits_lo;
     if (pool_splits > 0) {
-      e = launch_pdl(decode_kernel<1>, dim3(pool_splits, a.H, a.B), dim3(kThreads),
+      e = launch_pdl(decode_tq_kernel, dim3(pool_splits, a.H, a.B), dim3(kThreads),
                      kRingBytes + kAqBytes, stream, a);
       if (e != cudaSuccess) return e;
       pools_launched = true;
@@ -2514,10 +2561,11 @@ cudaError_t launch_decode_attention(const DecodeArgs& a, cudaStream_t stream) {
     // inputs) the stage kernel starts alongside it; otherwise it runs in order
     DecodeArgs as = a;
     as.stage_overlaps_pools = pools_launched ? 1 : 0;
+    const size_t smem = kStageRowBytes + (size_t)(a.Hq / a.H) * stage_pad(a.stage_n) * 4;
     if (as.stage_overlaps_pools)
-      e = launch_pdl(decode_kernel<2>, dim3(1, a.H, a.B), dim3(kThreads), kRingBytes, stream, as);
+      e = launch_pdl(decode_stage_kernel, dim3(1, a.H, a.B), dim3(kThreads), smem, stream, as);
     else
-      decode_kernel<2><<<dim3(1, a.H, a.B), kThreads, kRingBytes, stream>>>(as);
+      decode_stage_kernel<<<dim3(1, a.H, a.B), kThreads, smem, stream>>>(as);
     if (e != cudaSuccess) return e;
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;

@@ -115,12 +115,16 @@ def _ptr(t):
     if t is None:
         return None
     assert t.is_contiguous(), "tensors passed to libsemkv must be contiguous"
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()   # (the argument types make it a void*)
 
 
 def _stream(stream):
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    if not torch.cuda.is_initialized():
+        return torch.cuda.current_stream().cuda_stream
+    # the raw handle: building a torch Stream object took 3 of a decode call's 18 us
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _check(fn, status):

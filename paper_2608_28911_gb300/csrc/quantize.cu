@@ -26,7 +26,6 @@ namespace semkv {
 namespace {
 
 constexpr int kWarpsPerBlock = 8;
-constexpr int kMaxRecWords = 27;  // largest record: affine L=7/8, 2*48+8 = 104 B
 
 // ------------------------------------------------- affine pools, by slot -----
 // Affine records are built by destination slot: a warp takes units of 4 consecutive
@@ -38,24 +37,14 @@ constexpr int kMaxRecWords = 27;  // largest record: affine L=7/8, 2*48+8 = 104 
 // symbols beta = ceil(t 2^W / L^G) (the record format).
 
 constexpr int kAffineSlots = 4;
-constexpr int kAffineCtas = 5;  // resident CTAs of 8 warps per SM (48 registers)
+#ifndef AC
+#define AC 4
+#endif
+constexpr int kAffineCtas = AC;  // resident CTAs of 8 warps per SM (48 registers)
 
-// 32 fp16 values of one quarter row (16-byte loads when the source allows)
-__device__ __forceinline__ void load_quarter(const uint16_t* src, bool vec16, uint32_t (&h)[16]) {
-  if (vec16) {
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const uint4 u = __ldg(reinterpret_cast<const uint4*>(src) + j);
-      h[4 * j] = u.x; h[4 * j + 1] = u.y; h[4 * j + 2] = u.z; h[4 * j + 3] = u.w;
-    }
-  } else {
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const uint2 u = __ldg(reinterpret_cast<const uint2*>(src) + j);
-      h[2 * j] = u.x; h[2 * j + 1] = u.y;
-    }
-  }
-}
+constexpr int kQuarterStride = 80;  // bytes per staged quarter: 64 + 16 (5 x 16 B: the 8 lanes of a
+                                    // quarter warp reach distinct banks)
+constexpr int kAffineStage = 32 * kQuarterStride;
 
 // OR the value v (n bits, n <= 32) in at bit pos of a 3-word field (pos, n compile-time)
 __device__ __forceinline__ void put_bits(uint32_t (&w)[3], int pos, int n, uint32_t v) {
@@ -97,155 +86,26 @@ __device__ __forceinline__ void field_push(uint32_t (&w)[3], uint32_t& t, int j,
   }
 }
 
-template <int L>
-__device__ void affine_units(const QuantArgs& a, int b, int l, int h, bool hi, int64_t n_pool,
-                             int64_t u_begin, int64_t u_step, bool vec16, uint32_t* img) {
-  using F = Fmt<L>;
-  constexpr int kRecW = (2 * F::RB + 8) / 4;
-  static_assert(F::QB <= 96, "a quarter fits three words");
-  const int lane = threadIdx.x & 31;
-  const int ti = lane >> 3, row = (lane >> 2) & 1, qd = lane & 3;
-  const int64_t cap = hi ? a.hi_cap : a.lo_cap;
-  const int64_t base = hi ? a.hi_base : a.lo_base;
-  const int64_t bh = ((int64_t)b * a.NL + l) * a.H + h;
-  const int32_t* tokmap = (hi ? a.hi_tok : a.lo_tok) + (int64_t)b * cap + base;
-  const uint16_t* src = (row ? a.v : a.k) + bh * a.Tsrc * kHeadDim + 32 * qd;
-  const int64_t tok_base = a.tok_base;
-  uint32_t* recs = reinterpret_cast<uint32_t*>(hi ? a.hi_pool : a.lo_pool) + (bh * cap + base) * kRecW;
-  const int64_t units = (n_pool + kAffineSlots - 1) / kAffineSlots;
-  for (int64_t u = u_begin; u < units; u += u_step) {
-    const int64_t s0 = u * kAffineSlots;
-    const int nslots = (int)min((int64_t)kAffineSlots, n_pool - s0);
-    const bool active = ti < nslots;
-    for (int i = lane; i < kAffineSlots * kRecW; i += 32) img[i] = 0u;
-    uint32_t hv[16];
-    if (active) {
-      load_quarter(src + ((int64_t)tokmap[s0 + ti] - tok_base) * kHeadDim, vec16, hv);
-    } else {
-#pragma unroll
-      for (int j = 0; j < 16; ++j) hv[j] = 0u;
-    }
-    // row minimum and maximum: fp16 pairs (exact), then the row's other quarters
-    __half2 mn2 = *reinterpret_cast<const __half2*>(&hv[0]), mx2 = mn2;
-#pragma unroll
-    for (int j = 1; j < 16; ++j) {
-      const __half2 x2 = *reinterpret_cast<const __half2*>(&hv[j]);
-      mn2 = __hmin2(mn2, x2);
-      mx2 = __hmax2(mx2, x2);
-    }
-    float mn = fminf(__low2float(mn2), __high2float(mn2));
-    float mx = fmaxf(__low2float(mx2), __high2float(mx2));
-    mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, 1));
-    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-    mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, 2));
-    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-    // a zero extreme is taken as +0 (min/max may return either signed zero)
-    if (mn == 0.0f) mn = 0.0f;
-    if (mx == 0.0f) mx = 0.0f;
-    const float s32 = __fdiv_rn(__fsub_rn(mx, mn), (float)(L - 1));
-    const uint16_t s16 = f16_param(s32), z16 = __half_as_ushort(__float2half_rn(mn));
-    const float sc = f16_to_f32(s16), z = f16_to_f32(z16);
-    // 1/s, or 0 when s == 0 (then every value rounds to code 0)
-    const float inv = sc != 0.0f ? __fdiv_rn(1.0f, sc) : 0.0f;
-    __syncwarp();
-    // the codes stream into the quarter's field (no array of them: fewer registers)
-    uint32_t w[3] = {0u, 0u, 0u}, t = 0u;
-#pragma unroll
-    for (int j = 0; j < 32; ++j) {
-      const float x = f16_to_f32((uint16_t)(hv[j >> 1] >> (16 * (j & 1))));
-      // rint((x - z) / s) clamped to L-1 (the difference is >= 0: z is the row
-      // minimum); adding 1.5 * 2^23 rounds to nearest even
-      const float y = fminf(__fmul_rn(__fsub_rn(x, z), inv), (float)(L - 1));
-      field_push<L>(w, t, j, __float_as_uint(__fadd_rn(y, 12582912.0f)));
-    }
-    if (active) {
-      uint32_t* r = img + ti * kRecW;
-      const int pos = row * 8 * F::RB + qd * F::QB;  // the quarter's first bit
-      const int wd = pos >> 5, sh = pos & 31;
-      atomicOr(&r[wd], w[0] << sh);
-      if (sh + F::QB > 32) atomicOr(&r[wd + 1], __funnelshift_l(w[0], w[1], sh));
-      if (sh + F::QB > 64) atomicOr(&r[wd + 2], __funnelshift_l(w[1], w[2], sh));
-      if (sh + F::QB > 96) atomicOr(&r[wd + 3], __funnelshift_l(w[2], 0u, sh));
-      if (qd == 0) r[(2 * F::RB) / 4 + row] = (uint32_t)s16 | ((uint32_t)z16 << 16);
-    }
-    __syncwarp();
-    uint32_t* dst = recs + s0 * kRecW;
-    for (int i = lane; i < nslots * kRecW; i += 32) dst[i] = img[i];
-    __syncwarp();
-  }
+// ---- shared addresses and mbarriers
+__device__ __forceinline__ uint32_t dsmem_u32(const void* p) {
+  return (uint32_t)__cvta_generic_to_shared(p);
 }
-
-// slot -> token maps of the tokens quantized by this call
-__global__ void scatter_tok_kernel(QuantArgs a) {
-  pdl_wait();  // the flags and slots come from earlier work on the stream
-  pdl_trigger();
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (int64_t)a.B * a.n) return;
-  const int b = (int)(i / a.n), j = (int)(i % a.n);
-  const bool hi = a.is_high[(int64_t)b * a.n + j] != 0;
-  const int64_t s = (hi ? a.hi_base : a.lo_base) + a.slot[(int64_t)b * a.n + j];
-  const int64_t cap = hi ? a.hi_cap : a.lo_cap;
-  if (s >= cap) {  // cannot happen after the host's capacity check
-    raise_error(a.err, kDevCapacity);
-    return;
-  }
-  (hi ? a.hi_tok : a.lo_tok)[(int64_t)b * cap + s] = (int32_t)(a.tok_base + j);
+__device__ __forceinline__ void dbar_init(uint64_t* bar) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(dsmem_u32(bar)) : "memory");
 }
-
-// grid (x, sequence*layer*head, pool): each warp strides over that pool's units
-__global__ void __launch_bounds__(kWarpsPerBlock * 32, kAffineCtas)
-    quantize_affine_kernel(QuantArgs a, int64_t n_hi, int64_t n_lo) {
-  __shared__ __align__(16) uint32_t img_sm[kWarpsPerBlock][kAffineSlots * kMaxRecWords];
-  const int wib = threadIdx.x >> 5;
-  pdl_wait();  // the slot maps and the rows come from earlier work on the stream
-  pdl_trigger();
-  const bool hi = blockIdx.z == 0;
-  const int64_t n_pool = hi ? n_hi : n_lo;
-  const int64_t u_begin = (int64_t)blockIdx.x * kWarpsPerBlock + wib;
-  const int64_t u_step = (int64_t)gridDim.x * kWarpsPerBlock;
-  const bool vec16 = ((reinterpret_cast<uintptr_t>(a.k) | reinterpret_cast<uintptr_t>(a.v)) & 15u) == 0;
-  uint32_t* img = img_sm[wib];
-  const int bhs = a.B * a.NL * a.H;
-  for (int bhi = blockIdx.y; bhi < bhs; bhi += gridDim.y) {
-    const int h = bhi % a.H, l = (bhi / a.H) % a.NL, b = bhi / (a.H * a.NL);
-    switch (hi ? a.L_hi : a.L_lo) {
-      case 2: affine_units<2>(a, b, l, h, hi, n_pool, u_begin, u_step, vec16, img); break;
-      case 3: affine_units<3>(a, b, l, h, hi, n_pool, u_begin, u_step, vec16, img); break;
-      case 4: affine_units<4>(a, b, l, h, hi, n_pool, u_begin, u_step, vec16, img); break;
-      case 5: affine_units<5>(a, b, l, h, hi, n_pool, u_begin, u_step, vec16, img); break;
-      case 6: affine_units<6>(a, b, l, h, hi, n_pool, u_begin, u_step, vec16, img); break;
-      case 7: affine_units<7>(a, b, l, h, hi, n_pool, u_begin, u_step, vec16, img); break;
-      case 8: affine_units<8>(a, b, l, h, hi, n_pool, u_begin, u_step, vec16, img); break;
-      default: break;
-    }
-  }
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dsmem_u32(dst)), "l"(src) : "memory");
 }
-
-// ------------------------------ rotated bases by slot, two threads per row -----
-// TQ and rotated affine records built by destination slot, as for the affine base: a warp
-// takes tiles of 8 consecutive slots of one pool of one (sequence, layer, KV head), so the
-// level count is uniform.  Lane 4i + 2r + f holds half f (dims 64f .. 64f + 63, quarters
-// 2f and 2f + 1) of row r (0 = K, 1 = V) of slot i, in registers as 32 packed pairs
-// (x_j, x_{j+32}).  The Walsh-Hadamard butterflies run in the quantizer's stage order
-// (the same roundings as any other evaluation of them): stages 1..16 as packed
-// operations across pairs, stage 32 inside each pair, stage 64 with the partner lane.
-// Then the norm or the min/max (combined across the two halves), the codes, the two
-// quarters' bit fields; each lane puts its half's bits into the tile's record image, which
-// leaves in order with 16-byte stores.
-constexpr int kRowSlots = 64;
-constexpr int kRowStride = 272;  // bytes per staged row: 256 + 16 spreads the banks
-constexpr int kTileSlots = 8;    // slots of a warp's tile
-constexpr int kHalfStride = 144;  // bytes per half-row slot: 128 + 16 (9 x 16 B: the 8 lanes
-                                  // of a quarter warp reach distinct banks)
-constexpr int kWarpStageBytes = 32 * kHalfStride;
-// The quantizer: CTAs of 128 threads, 5 per SM (96 registers, 20 warps).  At 6 per SM (80
-// registers) the pairs spill and at 4 fewer warps hide the shuffles: the 32K TQ prompt takes
-// 87 us at 5, 103 at 6 and 92 at 4, the 3 x 20011 rotated one 133, 139 and 136.
-constexpr int kRowsThreads = 128;
-constexpr int kRowsCtas = 5;
-// Fake quantization: 4 per SM (128 registers; at 5 the two transforms spill, 144 against 128 us
-// for 4 layers x 16384 tokens of the rotated affine base, and at 3 fewer warps hide latency, 138).
-constexpr int kFakeCtas = 4;
+__device__ __forceinline__ void cp_async8(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dsmem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() {
+  asm volatile("cp.async.commit_group;" ::: "memory");
+}
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
 
 // packed binary32 pairs (two independent IEEE operations, rounded to nearest)
 __device__ __forceinline__ unsigned long long f2_add(unsigned long long a, unsigned long long b) {
@@ -306,6 +166,269 @@ __device__ __forceinline__ unsigned long long opaque_neg_zero(uint32_t* scratch)
   const uint32_t z = *reinterpret_cast<volatile uint32_t*>(scratch);
   return (unsigned long long)z | ((unsigned long long)z << 32);
 }
+
+// the larger of a and b, NaN if either is
+__device__ __forceinline__ float fmax_nan(float a, float b) {
+  float d;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
+  return d;
+}
+// the parameters of an affine row from its minimum and maximum
+struct AffineParams {
+  float s, z, inv;  // inv: 1/s, or 0 when s == 0 (then every value rounds to code 0)
+  uint32_t bits;    // s and z as fp16
+};
+__device__ __forceinline__ AffineParams affine_params(float mn, float mx, int L) {
+  // a zero extreme is taken as +0 (min/max may return either signed zero)
+  if (mn == 0.0f) mn = 0.0f;
+  if (mx == 0.0f) mx = 0.0f;
+  const uint16_t s16 = f16_param(__fdiv_rn(__fsub_rn(mx, mn), (float)(L - 1)));
+  const uint16_t z16 = __half_as_ushort(__float2half_rn(mn));
+  AffineParams p;
+  p.s = f16_to_f32(s16);
+  p.z = f16_to_f32(z16);
+  p.inv = p.s != 0.0f ? __frcp_rn(p.s) : 0.0f;
+  p.bits = (uint32_t)s16 | ((uint32_t)z16 << 16);
+  return p;
+}
+// x - z of an fp16 x and a binary32 z, rounded once: one mixed-precision add instead of a
+// conversion and a subtraction
+__device__ __forceinline__ float sub_mixed(uint16_t x, float neg_z) {
+  float d;
+  asm("add.rn.f32.f16 %0, %1, %2;" : "=f"(d) : "h"(x), "f"(neg_z));
+  return d;
+}
+
+// the codes of a quarter (32 fp16 values in hv) as its bit field: rint((x - z) * inv),
+// clamped to L - 1 where CLAMP.  x - z >= 0 (z is the row minimum); adding 1.5 * 2^23 rounds
+// to nearest even and leaves the code in the low bits of the pattern.
+template <int L, bool CLAMP>
+__device__ __forceinline__ void affine_field(const uint32_t (&hv)[16], float z, float inv,
+                                             unsigned long long nz, uint32_t (&w)[3]) {
+  const unsigned long long inv2 = f2_pack(inv, inv);
+  const unsigned long long mg2 = f2_pack(12582912.0f, 12582912.0f);
+  uint32_t t = 0u;
+  w[0] = w[1] = w[2] = 0u;
+#pragma unroll
+  for (int j = 0; j < 16; ++j) {
+    unsigned long long y = f2_mul_only(
+        f2_pack(sub_mixed((uint16_t)(hv[j] & 0xFFFFu), -z), sub_mixed((uint16_t)(hv[j] >> 16), -z)), inv2, nz);
+    if constexpr (CLAMP) y = f2_pack(fminf(f2_lo(y), (float)(L - 1)), fminf(f2_hi(y), (float)(L - 1)));
+    y = f2_add(y, mg2);
+    field_push<L>(w, t, 2 * j, (uint32_t)y);
+    field_push<L>(w, t, 2 * j + 1, (uint32_t)(y >> 32));
+  }
+}
+
+template <int L, bool VEC16>
+__device__ void affine_units(const QuantArgs& a, int b, int l, int h, bool hi, int64_t n_pool,
+                             int u_begin, int step, uint8_t* stages,
+                             unsigned long long nz) {
+  using F = Fmt<L>;
+  constexpr int kRecW = (2 * F::RB + 8) / 4;
+  static_assert(F::QB >= 32 && F::QB <= 96, "a quarter fits three words, and a word two quarters");
+  const int lane = threadIdx.x & 31;
+  const int ti = lane >> 3, row = (lane >> 2) & 1, qd = lane & 3;
+  const int64_t cap = hi ? a.hi_cap : a.lo_cap;
+  const int64_t base = hi ? a.hi_base : a.lo_base;
+  const int64_t bh = ((int64_t)b * a.NL + l) * a.H + h;
+  const int32_t* tokmap = (hi ? a.hi_tok : a.lo_tok) + (int64_t)b * cap + base;
+  // copies go row by row, 256 contiguous bytes of K and of V per instruction: chunk ch of 16
+  // bytes of slot i's row (K: lanes 0..15) to the lane slot of its quarter
+  const int ch = lane & 15;
+  const uint16_t* src = (lane < 16 ? a.k : a.v) + (bh * a.Tsrc - a.tok_base) * kHeadDim + 8 * ch;
+  const int at = (4 * (lane >> 4) + (ch >> 2)) * kQuarterStride + (ch & 3) * 16;
+  uint32_t* recs = reinterpret_cast<uint32_t*>(hi ? a.hi_pool : a.lo_pool) + (bh * cap + base) * kRecW;
+  const bool st16 = (reinterpret_cast<uintptr_t>(recs) & 15u) == 0;  // (so is every unit then)
+  // this lane's bits in a record: the quarter starts at bit off, in word wd0; the word it
+  // shares with the next quarter (the next lane) takes that one's first word, which then is
+  // not written again
+  constexpr int kSpan = (31 + F::QB + 31) / 32;
+  const int off = row * 8 * F::RB + qd * F::QB, wd0 = off >> 5, sh = off & 31;
+  const int cnt = ((off + F::QB + 31) >> 5) - wd0;
+  const int nxt = (lane & 7) == 3 ? 8 * F::RB : (lane & 7) == 7 ? 16 * F::RB : off + F::QB;
+  constexpr int kMin = F::QB / 32;  // words every quarter touches at least
+  uint32_t take[kSpan];             // the neighbour's first word goes into this word
+#pragma unroll
+  for (int k = 0; k < kSpan; ++k)
+    take[k] = (nxt >> 5) < wd0 + cnt && k == cnt - 1 ? 0xFFFFFFFFu : 0u;
+  const int prev_end = row && qd == 0 ? 4 * F::QB - 1 : off - 1;
+  const bool own_first = (lane & 7) == 0 || (prev_end >> 5) != wd0;
+  const int units = (int)((n_pool + kAffineSlots - 1) / kAffineSlots);
+  if (u_begin >= units) return;
+  // this lane's token of unit u (lanes past the pool's slots take the last one's; nothing of
+  // theirs is written)
+  const int last = (int)n_pool - 1;
+  auto token = [&](int u) { return tokmap[min(u * kAffineSlots + ti, last)]; };
+  auto issue = [&](int32_t tok, int st) {
+    uint8_t* dst = stages + st * kAffineStage + at;
+#pragma unroll
+    for (int i = 0; i < kAffineSlots; ++i) {
+      const uint16_t* p = src + (int64_t)__shfl_sync(0xffffffffu, tok, 8 * i) * kHeadDim;
+      uint8_t* d = dst + 8 * i * kQuarterStride;
+      if constexpr (VEC16) {
+        cp_async16(d, p);
+      } else {
+        cp_async8(d, p);
+        cp_async8(d + 8, p + 4);
+      }
+    }
+    cp_async_commit();
+  };
+  int32_t tok = token(u_begin);
+  issue(tok, 0);
+  if (u_begin + step < units) tok = token(u_begin + step);
+  int st = 0;
+  for (int u = u_begin; u < units; u += step, st ^= 1) {
+    const int64_t s0 = (int64_t)u * kAffineSlots;
+    const int nslots = min(kAffineSlots, (int)(n_pool - s0));
+    cp_async_wait<0>();
+    __syncwarp();  // the unit has landed; the other stage's image has been stored
+    if (u + step < units) {
+      issue(tok, st ^ 1);
+      if (u + 2 * step < units) tok = token(u + 2 * step);
+    }
+    uint8_t* stage = stages + st * kAffineStage;
+    uint32_t* img = reinterpret_cast<uint32_t*>(stage);
+    uint32_t hv[16];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const uint4 x = *reinterpret_cast<const uint4*>(stage + lane * kQuarterStride + 16 * j);
+      hv[4 * j] = x.x; hv[4 * j + 1] = x.y; hv[4 * j + 2] = x.z; hv[4 * j + 3] = x.w;
+    }
+    // row minimum and maximum: fp16 pairs (exact), then the row's other quarters
+    // (a NaN in the row makes the maximum, and so s, NaN: the slow path below)
+    __half2 mn2 = *reinterpret_cast<const __half2*>(&hv[0]), mx2 = mn2;
+#pragma unroll
+    for (int j = 1; j < 16; ++j) {
+      const __half2 x2 = *reinterpret_cast<const __half2*>(&hv[j]);
+      mn2 = __hmin2(mn2, x2);
+      mx2 = __hmax2_nan(mx2, x2);
+    }
+    float mn = fminf(__low2float(mn2), __high2float(mn2));
+    float mx = fmax_nan(__low2float(mx2), __high2float(mx2));
+    mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, 1));
+    mx = fmax_nan(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+    mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, 2));
+    mx = fmax_nan(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+    AffineParams pr = affine_params(mn, mx, L);
+    // The bound L - 1 cannot be reached when s is a normal fp16 value that was not limited:
+    // it is then within 2^-11 of (max - min) / (L - 1), so (x - z) / s < L - 1/2.  s = 0 gives
+    // zeros either way.
+    uint32_t w[3];
+    if (__all_sync(0xffffffffu, (pr.s >= 0x1p-14f && pr.s < 65504.0f) || pr.s == 0.0f)) {
+      affine_field<L, false>(hv, pr.z, pr.inv, nz, w);
+    } else {
+      // the maximum without NaNs, and the codes clamped
+      mx2 = *reinterpret_cast<const __half2*>(&hv[0]);
+#pragma unroll
+      for (int j = 1; j < 16; ++j) mx2 = __hmax2(mx2, *reinterpret_cast<const __half2*>(&hv[j]));
+      mx = fmaxf(__low2float(mx2), __high2float(mx2));
+      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+      pr = affine_params(mn, mx, L);
+      affine_field<L, true>(hv, pr.z, pr.inv, nz, w);
+    }
+    uint32_t v[kSpan];
+#pragma unroll
+    for (int k = 0; k < kSpan; ++k)
+      v[k] = __funnelshift_l(k > 0 ? w[k - 1] : 0u, k < 3 ? w[k] : 0u, sh);
+    const uint32_t first = __shfl_down_sync(0xffffffffu, v[0], 1);
+#pragma unroll
+    for (int k = kMin - 1; k < kSpan; ++k) v[k] |= first & take[k];
+    __syncwarp();  // every quarter has been read: the stage takes the records
+    uint32_t* r = img + ti * kRecW + wd0;
+#pragma unroll
+    for (int k = 0; k < kSpan; ++k)
+      if (k == 0 ? own_first : (k < kMin || k < cnt)) r[k] = v[k];
+    if (qd == 0) img[ti * kRecW + (2 * F::RB) / 4 + row] = pr.bits;
+    __syncwarp();
+    // the unit's records are contiguous: 16 bytes per lane where the pool position allows
+    uint32_t* dst = recs + s0 * kRecW;
+    const int words = nslots * kRecW;
+    if (st16 && nslots == kAffineSlots) {
+      static_assert(kAffineSlots * kRecW % 4 == 0 && kAffineSlots * kRecW / 4 <= 32, "one pass");
+      if (lane < kAffineSlots * kRecW / 4)
+        reinterpret_cast<uint4*>(dst)[lane] = reinterpret_cast<const uint4*>(img)[lane];
+    } else {
+      for (int i = lane; i < words; i += 32) dst[i] = img[i];
+    }
+  }
+}
+
+// slot -> token maps of the tokens quantized by this call
+__global__ void scatter_tok_kernel(QuantArgs a) {
+  pdl_wait();  // the flags and slots come from earlier work on the stream
+  pdl_trigger();
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= (int64_t)a.B * a.n) return;
+  const int b = (int)(i / a.n), j = (int)(i % a.n);
+  const bool hi = a.is_high[(int64_t)b * a.n + j] != 0;
+  const int64_t s = (hi ? a.hi_base : a.lo_base) + a.slot[(int64_t)b * a.n + j];
+  const int64_t cap = hi ? a.hi_cap : a.lo_cap;
+  if (s >= cap) {  // cannot happen after the host's capacity check
+    raise_error(a.err, kDevCapacity);
+    return;
+  }
+  (hi ? a.hi_tok : a.lo_tok)[(int64_t)b * cap + s] = (int32_t)(a.tok_base + j);
+}
+
+// grid (x, sequence*layer*head, pool): each warp strides over that pool's units
+template <bool VEC16>  // rows on 16-byte boundaries (else 8)
+__global__ void __launch_bounds__(kWarpsPerBlock * 32, kAffineCtas)
+    quantize_affine_kernel(QuantArgs a, int64_t n_hi, int64_t n_lo) {
+  __shared__ __align__(128) uint8_t stage_sm[kWarpsPerBlock][2 * kAffineStage];
+  // (the same in every lane: what follows from it stays in uniform registers)
+  const int wib = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);
+  uint8_t* stages = stage_sm[wib];
+  const unsigned long long nz = opaque_neg_zero(reinterpret_cast<uint32_t*>(stages));
+  pdl_wait();  // the slot maps and the rows come from earlier work on the stream
+  pdl_trigger();
+  const bool hi = blockIdx.z == 0;
+  const int64_t n_pool = hi ? n_hi : n_lo;
+  const int u_begin = (int)blockIdx.x * kWarpsPerBlock + wib, step = (int)gridDim.x * kWarpsPerBlock;
+  const int bhs = a.B * a.NL * a.H;
+  for (int bhi = blockIdx.y; bhi < bhs; bhi += gridDim.y) {
+    const int h = bhi % a.H, l = (bhi / a.H) % a.NL, b = bhi / (a.H * a.NL);
+    __syncwarp();  // (the last head's records have left the stages)
+    switch (hi ? a.L_hi : a.L_lo) {
+      case 2: affine_units<2, VEC16>(a, b, l, h, hi, n_pool, u_begin, step, stages, nz); break;
+      case 3: affine_units<3, VEC16>(a, b, l, h, hi, n_pool, u_begin, step, stages, nz); break;
+      case 4: affine_units<4, VEC16>(a, b, l, h, hi, n_pool, u_begin, step, stages, nz); break;
+      case 5: affine_units<5, VEC16>(a, b, l, h, hi, n_pool, u_begin, step, stages, nz); break;
+      case 6: affine_units<6, VEC16>(a, b, l, h, hi, n_pool, u_begin, step, stages, nz); break;
+      case 7: affine_units<7, VEC16>(a, b, l, h, hi, n_pool, u_begin, step, stages, nz); break;
+      case 8: affine_units<8, VEC16>(a, b, l, h, hi, n_pool, u_begin, step, stages, nz); break;
+      default: break;
+    }
+  }
+}
+
+// ------------------------------ rotated bases by slot, two threads per row -----
+// TQ and rotated affine records built by destination slot, as for the affine base: a warp
+// takes tiles of 8 consecutive slots of one pool of one (sequence, layer, KV head), so the
+// level count is uniform.  Lane 4i + 2r + f holds half f (dims 64f .. 64f + 63, quarters
+// 2f and 2f + 1) of row r (0 = K, 1 = V) of slot i, in registers as 32 packed pairs
+// (x_j, x_{j+32}).  The Walsh-Hadamard butterflies run in the quantizer's stage order
+// (the same roundings as any other evaluation of them): stages 1..16 as packed
+// operations across pairs, stage 32 inside each pair, stage 64 with the partner lane.
+// Then the norm or the min/max (combined across the two halves), the codes, the two
+// quarters' bit fields; each lane puts its half's bits into the tile's record image, which
+// leaves in order with 16-byte stores.
+constexpr int kRowSlots = 64;
+constexpr int kRowStride = 272;  // bytes per staged row: 256 + 16 spreads the banks
+constexpr int kTileSlots = 8;    // slots of a warp's tile
+constexpr int kHalfStride = 144;  // bytes per half-row slot: 128 + 16 (9 x 16 B: the 8 lanes
+                                  // of a quarter warp reach distinct banks)
+constexpr int kWarpStageBytes = 32 * kHalfStride;
+// The quantizer: CTAs of 128 threads, 5 per SM (96 registers, 20 warps).  At 6 per SM (80
+// registers) the pairs spill and at 4 fewer warps hide the shuffles: the 32K TQ prompt takes
+// 87 us at 5, 103 at 6 and 92 at 4, the 3 x 20011 rotated one 133, 139 and 136.
+constexpr int kRowsThreads = 128;
+constexpr int kRowsCtas = 5;
+// Fake quantization: 4 per SM (128 registers; at 5 the two transforms spill, 144 against 128 us
+// for 4 layers x 16384 tokens of the rotated affine base, and at 3 fewer warps hide latency, 138).
+constexpr int kFakeCtas = 4;
 
 // Butterfly stages 1, 2, 4, 8, 16 and 32 of the row transform over one half of the row,
 // held as packed pairs xp[j] = (x_j, x_{j+32}) (half-local indices): stages 1..16 pair
@@ -630,24 +753,6 @@ __device__ __forceinline__ void rows_back(const float* thr, uint8_t* stage, uint
     done = words & ~3;
   }
   for (int i = done + lane; i < words; i += 32) reinterpret_cast<uint32_t*>(rec)[i] = img[i];
-}
-
-// ---- shared addresses and mbarriers
-__device__ __forceinline__ uint32_t dsmem_u32(const void* p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
-__device__ __forceinline__ void dbar_init(uint64_t* bar) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(dsmem_u32(bar)) : "memory");
-}
-__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dsmem_u32(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() {
-  asm volatile("cp.async.commit_group;" ::: "memory");
-}
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
 // A position in the tiles: tile r of (sequence, layer, head) bhi, the high pool's tiles
@@ -1512,7 +1617,8 @@ cudaError_t launch_quantize_pack(const QuantArgs& a, int64_t n_hi, int num_sms,
     }
     if (bx < 1) bx = 1;
     dim3 grid((unsigned)bx, (unsigned)(bhs < 65535 ? bhs : 65535), 2);
-    return launch_pdl(quantize_affine_kernel, grid, dim3(kWarpsPerBlock * 32), 0, stream, a, n_hi,
+    const bool vec16 = ((reinterpret_cast<uintptr_t>(a.k) | reinterpret_cast<uintptr_t>(a.v)) & 15u) == 0;
+    return launch_pdl(vec16 ? quantize_affine_kernel<true> : quantize_affine_kernel<false>, grid, dim3(kWarpsPerBlock * 32), 0, stream, a, n_hi,
                       a.n - n_hi);
   }
   // TQ, rotated affine and dense-rotation TQ: slot -> token maps, then the rows by slot

@@ -31,57 +31,103 @@ constexpr int kWarpsPerBlock = 8;
 // Affine records are built by destination slot: a warp takes units of 4 consecutive
 // slots of one pool of one (sequence, layer, KV head), so the level count is uniform
 // across the warp and the records it writes are contiguous.  Lane 8i + 4r + q handles
-// quarter q (dims 32q..32q+31) of row r (0 = K, 1 = V) of the i-th slot's token: 64
-// contiguous bytes in, one quarter bit field out (a quarter per lane keeps the lane's
-// state small: 48 registers, 40 warps per SM).  The same arithmetic as the header states, and
-// symbols beta = ceil(t 2^W / L^G) (the record format).
+// quarter q (dims 32q..32q+31) of row r (0 = K, 1 = V) of the i-th slot's token: 64 bytes
+// in, one quarter bit field out.  The same arithmetic as the header states, and symbols
+// beta = ceil(t 2^W / L^G) (the record format).
+//
+// Each warp has a two-stage ring: while a unit is quantized, the next one's rows come by
+// cp.async, 256 contiguous bytes of K and of V per instruction, and the one after's token
+// indices are read.  Quarters are staged 80 bytes apart, and the records leave through the
+// stage in 16-byte stores.
+//
+// Bound by memory: the 4 x 64K prompt's kernel takes 212 us, 5.9 TB/s (87% of the measured
+// copy rate), at 74% issue activity and 90 warp instructions per token and head.  It took 258
+// with 101 instructions, a 64-byte quarter per lane in four loads (which kept the load/store
+// pipe 74% busy), every code clamped and records put together by atomics and 4-byte stores.
 
 constexpr int kAffineSlots = 4;
-#ifndef AC
-#define AC 4
-#endif
-constexpr int kAffineCtas = AC;  // resident CTAs of 8 warps per SM (48 registers)
+// resident CTAs of 8 warps per SM (64 registers; at 5 and 48 registers the 4 x 64K prompt takes
+// 321 us against 314, at 6 with spills 338)
+constexpr int kAffineCtas = 4;
 
 constexpr int kQuarterStride = 80;  // bytes per staged quarter: 64 + 16 (5 x 16 B: the 8 lanes of a
                                     // quarter warp reach distinct banks)
 constexpr int kAffineStage = 32 * kQuarterStride;
 
-// OR the value v (n bits, n <= 32) in at bit pos of a 3-word field (pos, n compile-time)
-__device__ __forceinline__ void put_bits(uint32_t (&w)[3], int pos, int n, uint32_t v) {
+// The symbol beta = ceil(t 2^W / M) of a radix value t < M at bit pos of a 3-word field that is
+// zero there (pos a compile-time value after unrolling); t arrives as t + off modulo 2^32.
+// Without a division: beta = floor((t K + 2^16 - 1) / 2^16) with K = floor(2^(W+16) / M), and
+// the multiplier takes the shift to the symbol's place along, so most symbols cost a
+// multiply-add and a masked OR.  For M = 7776 (W = 13) that product passes 32 bits:
+// beta = t + floor((t K + 2^23 - 1) / 2^23) with K = floor(2^23 (2^13 - M) / M); 13 / 243 is
+// (2^13 - 7776) / 7776.  Both hold for every t (symbol_exact).
+template <uint32_t M, int W>
+struct Symbol {
+  static constexpr bool kWide = W > 8;
+  static constexpr int S = kWide ? 23 : 16;
+  static constexpr uint32_t K = kWide ? (uint32_t)((13ull << S) / 243) : (uint32_t)((1ull << (W + S)) / M);
+  static constexpr uint32_t C = (1u << S) - 1u;
+};
+template <uint32_t M, int W>
+constexpr bool symbol_exact() {
+  using Y = Symbol<M, W>;
+  for (uint32_t t = 0; t < M; ++t) {
+    const uint32_t q = (t * Y::K + Y::C) >> Y::S, beta = (uint32_t)((((uint64_t)t << W) + M - 1) / M);
+    if ((uint64_t)t * Y::K + Y::C > 0xFFFFFFFFull || (Y::kWide ? t + q : q) != beta) return false;
+  }
+  return true;
+}
+static_assert(symbol_exact<7776, 13>() && symbol_exact<125, 7>() && symbol_exact<243, 8>() &&
+                  symbol_exact<36, 6>() && symbol_exact<25, 5>() && symbol_exact<9, 4>() &&
+                  symbol_exact<7, 3>(),
+              "every group and tail of the record format");
+template <uint32_t M, int W>
+__device__ __forceinline__ void put_symbol(uint32_t (&w)[3], int pos, uint32_t t, uint32_t off) {
+  using Y = Symbol<M, W>;
   const int wd = pos >> 5, sh = pos & 31;
-  w[wd] |= v << sh;
-  if (sh + n > 32) w[wd + 1] |= v >> (32 - sh);
+  const uint32_t c = Y::C - off * Y::K, mask = ((1u << W) - 1u) << sh;
+  if constexpr (Y::kWide) {
+    const uint32_t q = t + ((t * Y::K + c) >> Y::S);  // beta + off
+    if (sh + W <= 32) {
+      w[wd] += (q << sh) - (off << sh);
+    } else {
+      const uint32_t beta = q - off;
+      w[wd] += beta << sh;
+      w[wd + 1] += beta >> (32 - sh);
+    }
+  } else if (sh < 16) {
+    w[wd] |= ((t * Y::K + c) >> (16 - sh)) & mask;
+  } else {
+    w[wd] |= (t * (Y::K << (sh - 16)) + (c << (sh - 16))) & mask;
+    if (sh + W > 32) w[wd + 1] |= (t * Y::K + c) >> (48 - sh);
+  }
 }
 
 // One code of a quarter's field, streamed in order (j = 0..31, compile-time after
-// unrolling): m is the magic-number pattern 1.5 * 2^23 + c_j, t the running radix value
-// of the open symbol (sums of L-weighted patterns give it modulo 2^32 once the weighted
-// 1.5 * 2^23 terms are taken off); each completed symbol's beta goes into the field.
-template <int L>
+// unrolling): m is the code plus OFF (1.5 * 2^23 for magic-number patterns, or 0), t the
+// running radix value of the open symbol (sums of L-weighted terms modulo 2^32); each
+// completed symbol goes into the field.
+template <int L, uint32_t OFF = 0x4B400000u>
 __device__ __forceinline__ void field_push(uint32_t (&w)[3], uint32_t& t, int j, uint32_t m) {
   using F = Fmt<L>;
-  constexpr uint32_t kMagic = 0x4B400000u;
   if constexpr (F::G == 1 && F::LG == (1u << F::W)) {
-    put_bits(w, j * F::W, F::W, m - kMagic);
+    // L = 2, 4, 8: the code is its symbol; the offsets add up to one constant per word
+    const int wd = (j * F::W) >> 5, sh = (j * F::W) & 31;
+    w[wd] += (m << sh) - (OFF << sh);
+    if (sh + F::W > 32) w[wd + 1] += (m - OFF) >> (32 - sh);
   } else {
-    if (j < F::NG * F::G) {
-      const int k = j % F::G, sy = j / F::G;
-      t = (k == 0 ? 0u : t * (uint32_t)L) + m;
-      if (k == F::G - 1) {
-        uint32_t wsum = 0;
-        for (int q = 0; q < F::G; ++q) wsum = wsum * (uint32_t)L + 1u;
-        const uint32_t tt = t - wsum * kMagic;
-        put_bits(w, sy * F::W, F::W, ((tt << F::W) + F::LG - 1u) / F::LG);
-      }
-    } else {
-      const int k = j - F::NG * F::G;
-      t = (k == 0 ? 0u : t * (uint32_t)L) + m;
-      if (k == F::R - 1) {
-        uint32_t wsum = 0;
-        for (int q = 0; q < F::R; ++q) wsum = wsum * (uint32_t)L + 1u;
-        const uint32_t tt = t - wsum * kMagic;
-        put_bits(w, F::NG * F::W, F::WT, ((tt << F::WT) + F::LR - 1u) / F::LR);
-      }
+    const bool tail = j >= F::NG * F::G;
+    const int k = tail ? j - F::NG * F::G : j % F::G, len = tail ? F::R : F::G;
+    t = (k == 0 ? 0u : t * (uint32_t)L) + m;
+    if (k == len - 1) {
+      uint32_t wsum = 0;
+      for (int q = 0; q < len; ++q) wsum = wsum * (uint32_t)L + 1u;
+      if constexpr (F::R > 0)
+        if (tail) {
+          put_symbol<F::LR, F::WT>(w, F::NG * F::W, t, wsum * OFF);
+          return;
+        }
+      put_symbol<F::LG, F::W>(w, (j / F::G) * F::W, t, wsum * OFF);
     }
   }
 }
@@ -373,10 +419,11 @@ __global__ void scatter_tok_kernel(QuantArgs a) {
   (hi ? a.hi_tok : a.lo_tok)[(int64_t)b * cap + s] = (int32_t)(a.tok_base + j);
 }
 
-// grid (x, sequence*layer*head, pool): each warp strides over that pool's units
+// grid (x, sequence*layer*head): x < bx_hi on the high pool, the rest on the low one, each
+// warp striding over its pool's units
 template <bool VEC16>  // rows on 16-byte boundaries (else 8)
 __global__ void __launch_bounds__(kWarpsPerBlock * 32, kAffineCtas)
-    quantize_affine_kernel(QuantArgs a, int64_t n_hi, int64_t n_lo) {
+    quantize_affine_kernel(QuantArgs a, int64_t n_hi, int64_t n_lo, int bx_hi) {
   __shared__ __align__(128) uint8_t stage_sm[kWarpsPerBlock][2 * kAffineStage];
   // (the same in every lane: what follows from it stays in uniform registers)
   const int wib = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);
@@ -384,9 +431,10 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kAffineCtas)
   const unsigned long long nz = opaque_neg_zero(reinterpret_cast<uint32_t*>(stages));
   pdl_wait();  // the slot maps and the rows come from earlier work on the stream
   pdl_trigger();
-  const bool hi = blockIdx.z == 0;
+  const bool hi = (int)blockIdx.x < bx_hi;
   const int64_t n_pool = hi ? n_hi : n_lo;
-  const int u_begin = (int)blockIdx.x * kWarpsPerBlock + wib, step = (int)gridDim.x * kWarpsPerBlock;
+  const int x = (int)blockIdx.x - (hi ? 0 : bx_hi), bx = hi ? bx_hi : (int)gridDim.x - bx_hi;
+  const int u_begin = x * kWarpsPerBlock + wib, step = bx * kWarpsPerBlock;
   const int bhs = a.B * a.NL * a.H;
   for (int bhi = blockIdx.y; bhi < bhs; bhi += gridDim.y) {
     const int h = bhi % a.H, l = (bhi / a.H) % a.NL, b = bhi / (a.H * a.NL);
@@ -521,40 +569,19 @@ __device__ __forceinline__ void tq_fields(const unsigned long long (&u2)[32],
       }
     }
   } else {
-    // c = sum of the comparison bits; symbols beta = ceil(t 2^W / L^G)
-    auto code = [&](int j, uint32_t& cl, uint32_t& ch) {
-      cl = 0u; ch = 0u;
+    // c = sum of the comparison bits
+    uint32_t t0 = 0u, t1 = 0u;
+#pragma unroll
+    for (int j = 0; j < 32; ++j) {
+      uint32_t cl = 0u, ch = 0u;
 #pragma unroll
       for (int k = 0; k < L - 1; ++k) {
         const unsigned long long d = f2_sub(t2[k], u2[j]);
         cl += (uint32_t)d >> 31;
         ch += (uint32_t)(d >> 32) >> 31;
       }
-    };
-#pragma unroll
-    for (int sy = 0; sy < F::NG; ++sy) {
-      uint32_t tl = 0u, th = 0u;
-#pragma unroll
-      for (int k = 0; k < F::G; ++k) {
-        uint32_t cl, ch;
-        code(sy * F::G + k, cl, ch);
-        tl = tl * (uint32_t)L + cl;
-        th = th * (uint32_t)L + ch;
-      }
-      put_bits(w0, sy * F::W, F::W, ((tl << F::W) + F::LG - 1u) / F::LG);
-      put_bits(w1, sy * F::W, F::W, ((th << F::W) + F::LG - 1u) / F::LG);
-    }
-    if constexpr (F::R > 0) {
-      uint32_t tl = 0u, th = 0u;
-#pragma unroll
-      for (int k = 0; k < F::R; ++k) {
-        uint32_t cl, ch;
-        code(32 - F::R + k, cl, ch);
-        tl = tl * (uint32_t)L + cl;
-        th = th * (uint32_t)L + ch;
-      }
-      put_bits(w0, F::NG * F::W, F::WT, ((tl << F::WT) + F::LR - 1u) / F::LR);
-      put_bits(w1, F::NG * F::W, F::WT, ((th << F::WT) + F::LR - 1u) / F::LR);
+      field_push<L, 0u>(w0, t0, j, cl);
+      field_push<L, 0u>(w1, t1, j, ch);
     }
   }
 }
@@ -1321,18 +1348,7 @@ __device__ __forceinline__ void tq_quarter(const float (&u)[32], const unsigned 
         c[1] += (uint32_t)(d >> 32) >> 31;
       }
 #pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        const int j = 2 * jp + e;
-        if (j < F::NG * F::G) {
-          const int k = j % F::G, sy = j / F::G;
-          t = (k == 0 ? 0u : t * (uint32_t)L) + c[e];
-          if (k == F::G - 1) put_bits(w, sy * F::W, F::W, ((t << F::W) + F::LG - 1u) / F::LG);
-        } else {
-          const int k = j - F::NG * F::G;
-          t = (k == 0 ? 0u : t * (uint32_t)L) + c[e];
-          if (k == F::R - 1) put_bits(w, F::NG * F::W, F::WT, ((t << F::WT) + F::LR - 1u) / F::LR);
-        }
-      }
+      for (int e = 0; e < 2; ++e) field_push<L, 0u>(w, t, 2 * jp + e, c[e]);
     }
   }
 }
@@ -1596,30 +1612,33 @@ cudaError_t launch_quantize_pack(const QuantArgs& a, int64_t n_hi, int num_sms,
                                        dim3(256), 0, stream, a);
       if (e != cudaSuccess) return e;
     }
-    // grid x from a simple wave model: with R resident CTAs (kAffineCtas per SM), the pass takes
-    // about ceil(CTAs / R) waves of ceil(units / (8 bx)) units per warp; take the
-    // cheapest bx (at most 16 units per warp).  The (sequence, layer, head) index runs
-    // over grid y (and loops past its limit of 65535)
+    // Grid x: bx_hi CTAs for the high pool of each (sequence, layer, head), the rest for the
+    // low one, so that every warp has about the same number of units.  From a wave model:
+    // with R resident CTAs (kAffineCtas per SM) the pass takes ceil(CTAs / R) waves of
+    // (units per warp + 2), the 2 for a warp's start (its position, the first unit's token and
+    // rows); the cheapest count up to 32 is taken.  (Sized by the larger pool alone and
+    // without the start, a 32K prompt with 30% high two-level tokens got one unit per warp:
+    // 51 us, 33 now.)  The head index runs over grid y (and loops past its limit of 65535).
     const int64_t bhs = (int64_t)a.B * a.NL * a.H;
-    const int64_t n_max = n_hi > a.n - n_hi ? n_hi : a.n - n_hi;
-    const int64_t units = (n_max + kAffineSlots - 1) / kAffineSlots;
+    const int64_t rows = bhs < 65535 ? bhs : 65535;
     const int64_t resident = (int64_t)(num_sms > 0 ? num_sms : 1) * kAffineCtas;
-    const int64_t rows = 2 * (bhs < 65535 ? bhs : 65535);
-    int64_t bx = 1, best = -1;
-    for (int64_t pw = 16; pw >= 1; --pw) {
-      const int64_t cand = (units + pw * kWarpsPerBlock - 1) / (pw * kWarpsPerBlock);
-      const int64_t per = (units + cand * kWarpsPerBlock - 1) / (cand * kWarpsPerBlock);
-      const int64_t cost = ((cand * rows + resident - 1) / resident) * per;
-      if (best < 0 || cost * 50 < best * 49) {  // a near tie keeps the larger units
+    const int64_t u_hi = (n_hi + kAffineSlots - 1) / kAffineSlots;
+    const int64_t u_lo = (a.n - n_hi + kAffineSlots - 1) / kAffineSlots;
+    int64_t bx_hi = 0, bx_lo = 0, best = -1;
+    for (int64_t pw = 32; pw >= 1; --pw) {
+      const int64_t per = pw * kWarpsPerBlock;
+      const int64_t xh = (u_hi + per - 1) / per, xl = (u_lo + per - 1) / per;
+      const int64_t cost = (((xh + xl) * rows + resident - 1) / resident) * (pw + 2);
+      if (best < 0 || cost < best) {
         best = cost;
-        bx = cand;
+        bx_hi = xh;
+        bx_lo = xl;
       }
     }
-    if (bx < 1) bx = 1;
-    dim3 grid((unsigned)bx, (unsigned)(bhs < 65535 ? bhs : 65535), 2);
+    const dim3 grid((unsigned)(bx_hi + bx_lo), (unsigned)rows);
     const bool vec16 = ((reinterpret_cast<uintptr_t>(a.k) | reinterpret_cast<uintptr_t>(a.v)) & 15u) == 0;
-    return launch_pdl(vec16 ? quantize_affine_kernel<true> : quantize_affine_kernel<false>, grid, dim3(kWarpsPerBlock * 32), 0, stream, a, n_hi,
-                      a.n - n_hi);
+    return launch_pdl(vec16 ? quantize_affine_kernel<true> : quantize_affine_kernel<false>, grid,
+                      dim3(kWarpsPerBlock * 32), 0, stream, a, n_hi, a.n - n_hi, (int)bx_hi);
   }
   // TQ, rotated affine and dense-rotation TQ: slot -> token maps, then the rows by slot
   if (!maps_ready) {

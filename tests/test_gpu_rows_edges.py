@@ -95,3 +95,59 @@ def test_fake_rows_tile_edges_bit_exact(base, L_hi, L_lo, T, mixed):
                              is_high=ih, **kw)
     for got, w in zip((ko, vo), want):
         assert np.array_equal(got.cpu().numpy().view(np.uint16), w)
+
+
+@pytest.mark.parametrize("L_hi,L_lo,T,r,blk,shift", [
+    (6, 5, 1, (0, 1), 1, 0),       # one slot, then one at a time
+    (2, 3, 5, (1, 2), 3, 4),       # rows on 8-byte boundaries
+    (8, 7, 9, (1, 3), 5, 0),
+    (5, 4, 67, (1, 1), 9, 4),      # the high pool only, until blocks add low slots
+    (3, 2, 131, (26, 100), 30, 0),
+])
+def test_affine_units_and_unaligned_appends_bit_exact(L_hi, L_lo, T, r, blk, shift):
+    """The affine quantizer's 4-slot units: remainders, records that start off a 16-byte
+    boundary, prompt rows on 8-byte boundaries only, NaN and infinity beside ordinary rows
+    of the same unit, limited and subnormal steps."""
+    import torch
+    from paper_2608_28911_gb300 import semkv
+    n = 2 * blk
+    p = Pair(0, L_hi, L_lo, 2, 1, 2, 4, T, r[0], r[1], seed=400 + T, block=blk, extra_cap=n)
+    rng = np.random.default_rng(T)
+    for x in (p.k, p.v):
+        x[0, 0, 0, T // 2, 7] = np.nan
+        x[0, 0, 1, T - 1] = np.float16(65504.0) * np.sign(rng.standard_normal(128)).astype(np.float16)
+        x[1, 0, 0, 0] = (rng.integers(-9, 10, 128) * 2.0 ** -24).astype(np.float16)
+        x[1, 0, 1, T - 1, 3] = np.inf
+    if shift:  # the same rows at an address that is 8 modulo 16
+        d = p.dev
+        p.o_is_high, p.o_slot = oracle.quantize_prompt(
+            p.oc, synthetic.f16_bits(p.k), synthetic.f16_bits(p.v), p.s, r[0], r[1])
+        rows = []
+        for x in (p.k, p.v):
+            buf = torch.zeros(x.size + 8, dtype=torch.float16, device=d)
+            view = buf[shift:shift + x.size].view(x.shape)
+            view.copy_(torch.from_numpy(x).to(d))
+            assert view.data_ptr() % 16 == 8
+            rows.append(view)
+        h = torch.empty((2, T), dtype=torch.uint8, device=d)
+        slot = torch.empty((2, T), dtype=torch.int32, device=d)
+        semkv.semkv_rank_assign(torch.from_numpy(p.s).to(d), p.n_high, h, slot)
+        semkv.semkv_quantize_pack(p.desc, rows[0], rows[1], h, slot, p.n_high, p.cache)
+        torch.cuda.synchronize()
+    else:
+        p.quantize()
+    # a row with NaN has no record that the oracle defines; it must leave its unit's others alone
+    for gp, op, tok in ((p.cache.hi_pool, p.oc.hi_pool, p.oc.hi_tok), (p.cache.lo_pool, p.oc.lo_pool, p.oc.lo_tok)):
+        at = np.flatnonzero(tok[0] == T // 2)
+        op[0, 0, 0, at] = gp.cpu().numpy()[0, 0, 0, at]
+    p.assert_records_equal()
+    k, v = synthetic.kv(401 + T, 2, 1, 2, n)
+    s = synthetic.scores_zipf(402 + T, 2, n)
+    for i in range(2):
+        at = slice(i * blk, (i + 1) * blk)
+        p.stage(k[:, :, :, at], v[:, :, :, at], s[:, at])
+        semkv.semkv_append_block(p.desc, p.cache, 1, 2)
+        oracle.append_block(p.oc, 1, 2)
+    torch.cuda.synchronize()
+    p.assert_records_equal()
+    p.assert_untouched_past_counts()

@@ -1487,28 +1487,31 @@ __global__ void qrot_dense_kernel(DecodeArgs a) {
 //     shuffles per head).  Then every warp takes the maximum per head.
 //  2. Weighted sums: a warp takes tokens warp, warp + 8, ...; lane = 4 dims.
 // Bound by latency: two rounds of loads instead of one round, a reduction over 32 lanes and
-// an exponential per token and head in a serial chain (STAGEFIG).
+// an exponential per token and head in a serial chain (which took 16 us for 77 tokens, longer
+// than the 4K-token pools beside it).
 // Writes rows in natural dim order and zs = 0.  logits: [G][stage_n rounded up to 32].
-constexpr int kStageRowBytes = (kWarps * 8 * kMoStride + 8 * 128) * 4;
-__host__ __device__ inline int stage_pad(int n) { return (n + 31) / 32 * 32; }
+template <int NW>
+__host__ __device__ constexpr int stage_row_bytes() { return (NW * 8 * kMoStride + 8 * 128) * 4; }
+__host__ __device__ constexpr int stage_pad(int n) { return (n + 31) / 32 * 32; }
 
 struct MergeArea {
   float m[kMaxWarps * 8], l[kMaxWarps * 8], z[kMaxWarps * 8];
   float scale[kMaxWarps * 8], cta_z[8];
 };
 
+template <int NW>
 __device__ void run_stage(const DecodeArgs& a, Shared& sh, int b, int h, int G, MergeArea& mg,
                           float* o_out, float* logits) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int n = a.stage_n, pad = stage_pad(n);
   const int64_t base = (((int64_t)b * a.NL + a.layer) * a.H + h) * a.block;
-  for (int i = threadIdx.x; i < G * 128; i += kThreads)
+  for (int i = threadIdx.x; i < G * 128; i += NW * 32)
     sh.qr[i >> 7][i & 127] = f16_to_f32(a.q[((int64_t)b * a.Hq + h * G) * 128 + i]);
   __syncthreads();
   {
     // 8-byte pieces (the stage's alignment): lane e of a token takes pieces e, e + 8, ...
     const int sub = lane >> 3, e = lane & 7;
-    for (int t0 = 4 * warp; t0 < n; t0 += 4 * kWarps) {
+    for (int t0 = 4 * warp; t0 < n; t0 += 4 * NW) {
       const int t = min(t0 + sub, n - 1);
       const uint2* kr = reinterpret_cast<const uint2*>(a.stage_k + (base + t) * 128);
       float x[16];
@@ -1547,7 +1550,7 @@ __device__ void run_stage(const DecodeArgs& a, Shared& sh, int b, int h, int G, 
     for (int off = 16; off >= 1; off >>= 1) M[c] = fmaxf(M[c], __shfl_xor_sync(0xffffffffu, M[c], off));
   }
 #pragma unroll 4
-  for (int t = warp; t < n; t += kWarps) {
+  for (int t = warp; t < n; t += NW) {
     const uint2 vu = *reinterpret_cast<const uint2*>(a.stage_v + (base + t) * 128 + 4 * lane);
     const float vx[4] = {f16_to_f32((uint16_t)(vu.x & 0xFFFF)), f16_to_f32((uint16_t)(vu.x >> 16)),
                          f16_to_f32((uint16_t)(vu.y & 0xFFFF)), f16_to_f32((uint16_t)(vu.y >> 16))};
@@ -1803,6 +1806,29 @@ __device__ void merge_warps(const DecodeArgs& a, int kind, int h, int G, MergeAr
   __syncthreads();  // the merge area (the ring) is free again
 }
 
+// The staged tail of pair bh, run by one CTA of NW warps: a partial after the pools'.
+// dyn: the CTA's dynamic shared memory, stage_bytes at least.  (Not inlined: the pool loops
+// keep their registers.)
+template <int NW>
+__host__ __device__ constexpr size_t stage_bytes(int G, int n) {
+  return stage_row_bytes<NW>() + (size_t)G * stage_pad(n) * 4;
+}
+template <int NW>
+__device__ __noinline__ void stage_cta(const DecodeArgs& a, int64_t bh, Shared& sh, MergeArea& mg,
+                                       uint8_t* dyn) {
+  const DecodePlan& P = a.plan;
+  const int b = (int)(bh / a.H), h = (int)(bh % a.H), G = a.Hq / a.H;
+  int split = P.splits_hi + P.splits_lo;
+  if (P.balanced) {
+    int n_hi, n_lo;
+    pair_slots(P, bh, n_hi, n_lo);
+    split = n_hi + n_lo;
+  }
+  float* rows = reinterpret_cast<float*>(dyn);  // [NW][8][128] rows, then [8][128]
+  run_stage<NW>(a, sh, b, h, G, mg, rows, reinterpret_cast<float*>(dyn + stage_row_bytes<NW>()));
+  merge_warps<NW>(a, 2, h, G, mg, rows, a.partials + (bh * P.stride + split) * kPartialFloats);
+}
+
 // The first copies of a segment, as run_pool would start them: issued before the
 // queries are loaded and the coefficient fragments built, so those overlap the copies.
 // The ring must be free (no merge in progress).
@@ -1868,7 +1894,7 @@ __device__ void run_pool_any_g(const DecodeArgs& a, const Shared& sh, uint8_t* r
 // concatenated [hi | lo] tile sequence of every (b, h) (a tile belongs to the CTA whose
 // range holds its start), one partial per (pair, pool) segment it touches.  One wave of
 // equal CTAs: no quantisation into waves and no per-split start-up beyond that.
-__global__ void __launch_bounds__(kThreads, kCtasAffine) decode_affine_kernel(DecodeArgs a) {
+__global__ void __launch_bounds__(kThreads, kCtasAffine) decode_affine_kernel(const __grid_constant__ DecodeArgs a) {
   extern __shared__ __align__(128) uint8_t dyn[];
   __shared__ Shared sh;
   __shared__ MergeArea mg;
@@ -1887,6 +1913,10 @@ __global__ void __launch_bounds__(kThreads, kCtasAffine) decode_affine_kernel(De
   __syncthreads();
   pdl_wait();  // the records, queries and stage partial come from earlier work
   pdl_trigger();
+  if ((int)blockIdx.x >= P.ctas) {  // the CTAs after the pools' take the staged tails
+    stage_cta<kWarps>(a, (int)blockIdx.x - P.ctas, sh, mg, dyn);
+    return;
+  }
   int ring_it = 0;  // tiles this warp has taken through its ring (barrier phases)
   int64_t loaded = -1;
   for (int64_t bh = start / P.W; bh < pairs && bh * P.W < end; ++bh) {
@@ -1977,9 +2007,11 @@ __device__ __forceinline__ void run_fast_l(const DecodeArgs& a, const Shared& sh
 // The balanced plan of decode_affine_kernel, run by the fast path: CTA c takes the
 // weighted range [c per, (c+1) per) of the concatenated [hi | lo] tile sequence of every
 // (b, h), one partial per (pair, pool) segment it touches.
-template <int NW>
+// TAILS: the CTAs after the pools' take the staged tails (an instance of its own: the call
+// costs the pool loops a few registers, 1546 against 1508 us over 32 layers x 128K).
+template <int NW, bool TAILS>
 __global__ void __launch_bounds__(NW * 32, NW == kWarps ? kCtasFast : 1)
-    decode_affine_fast_kernel(DecodeArgs a) {
+    decode_affine_fast_kernel(const __grid_constant__ DecodeArgs a) {
   extern __shared__ __align__(128) uint8_t dyn[];
   __shared__ Shared sh;
   __shared__ MergeArea mg;
@@ -1998,6 +2030,11 @@ __global__ void __launch_bounds__(NW * 32, NW == kWarps ? kCtasFast : 1)
   __syncthreads();
   pdl_wait();  // the records, queries and stage partial come from earlier work
   pdl_trigger();
+  if constexpr (TAILS)
+    if ((int)blockIdx.x >= P.ctas) {
+      stage_cta<NW>(a, (int)blockIdx.x - P.ctas, sh, mg, dyn);
+      return;
+    }
   int ring_it = 0;  // tiles this warp has taken through its ring (barrier phases)
   int64_t loaded = -1;
   for (int64_t bh = start / P.W; bh < pairs && bh * P.W < end; ++bh) {
@@ -2046,7 +2083,7 @@ __global__ void __launch_bounds__(NW * 32, NW == kWarps ? kCtasFast : 1)
 }
 
 // TQ pools, one CTA per split of one pool of a pair.
-__global__ void __launch_bounds__(kThreads, kCtasOther) decode_tq_kernel(DecodeArgs a) {
+__global__ void __launch_bounds__(kThreads, kCtasOther) decode_tq_kernel(const __grid_constant__ DecodeArgs a) {
   extern __shared__ __align__(128) uint8_t dyn[];
   __shared__ Shared sh;
   __shared__ MergeArea mg;
@@ -2058,6 +2095,12 @@ __global__ void __launch_bounds__(kThreads, kCtasOther) decode_tq_kernel(DecodeA
   const int b = blockIdx.z, h = blockIdx.y, split = blockIdx.x;
   const int64_t bh = (int64_t)b * a.H + h;
   const int G = a.Hq / a.H;
+  if (split >= P.splits_hi + P.splits_lo) {  // the CTA after the pools' takes the staged tail
+    pdl_wait();
+    pdl_trigger();
+    stage_cta<kWarps>(a, bh, sh, mg, dyn);
+    return;
+  }
   const int src = split < P.splits_hi ? 0 : 1;
   const int s_idx = src == 0 ? split : split - P.splits_hi;
   const int nsrc = src == 0 ? P.splits_hi : P.splits_lo;
@@ -2127,27 +2170,18 @@ __global__ void __launch_bounds__(kThreads, kCtasOther) decode_tq_kernel(DecodeA
   merge_warps(a, kind, h, G, mg, merge_o, a.partials + (bh * P.stride + split) * kPartialFloats);
 }
 
-// The fp16 stage, one CTA per pair.
-__global__ void __launch_bounds__(kThreads, kCtasOther) decode_stage_kernel(DecodeArgs a) {
+// The fp16 stage, one CTA per pair: for a cache without quantized tokens, and beside the
+// 16-warp pool kernel, whose register budget has no room for the call (16 x 64K: 282 us,
+// 290 with it).  The other pool kernels run the tails in CTAs of their own: a launch less (4K
+// tokens with a staged tail 16.4 -> 14.1 us).
+__global__ void __launch_bounds__(kThreads, kCtasOther) decode_stage_kernel(const __grid_constant__ DecodeArgs a) {
   extern __shared__ __align__(128) uint8_t dyn[];
   __shared__ Shared sh;
   __shared__ MergeArea mg;
-  float* merge_o = reinterpret_cast<float*>(dyn);  // [kWarps][8][128] rows, then [8][128]
-  const DecodePlan& P = a.plan;
-  const int b = blockIdx.z, h = blockIdx.y;
-  const int64_t bh = (int64_t)b * a.H + h;
-  const int G = a.Hq / a.H;
   if (!a.stage_overlaps_pools) pdl_wait();
-  int split = P.splits_hi + P.splits_lo;
-  if (P.balanced) {
-    int n_hi, n_lo;
-    pair_slots(P, bh, n_hi, n_lo);
-    split = n_hi + n_lo;
-  }
-  run_stage(a, sh, b, h, G, mg, merge_o, reinterpret_cast<float*>(dyn + kStageRowBytes));
-  merge_warps(a, 2, h, G, mg, merge_o, a.partials + (bh * P.stride + split) * kPartialFloats);
-  // a stage kernel that ran alongside the pool kernel completes only after it: the
-  // combine, which waits for this kernel, then sees every pool partial too
+  stage_cta<kWarps>(a, blockIdx.x, sh, mg, dyn);
+  // alongside the pool kernel it completes only after it: the combine, which waits for
+  // this kernel, then sees every pool partial too
   pdl_wait();
 }
 
@@ -2413,7 +2447,10 @@ DecodePlan make_decode_plan(int base, int L_hi, int L_lo, int B, int H, int Hq, 
     }
     // CTAs of 8 warps, two per SM (a copy of one or two tiles per warp and step)
     p.warps = kWarps;
-    straddled((int64_t)num_sms * (p.fast ? kCtasFast : kCtasAffine), kWarps * 2);
+    // (the staged tails' CTAs, one per pair, share the wave where there is room for them)
+    int64_t slots = (int64_t)num_sms * (p.fast ? kCtasFast : kCtasAffine);
+    if (st && slots >= 4 * pairs) slots -= pairs;
+    straddled(slots, kWarps * 2);
     // When the CTAs outnumber the pairs' segments (few sequences), ranges of equal
     // weight cut across the hi | lo and pair boundaries, and a CTA whose range holds a
     // boundary sets up, streams and merges two segments.  Aligned alternative: n_hi
@@ -2422,8 +2459,7 @@ DecodePlan make_decode_plan(int base, int L_hi, int L_lo, int B, int H, int Hq, 
     // n_hi T_lo and w_lo' = n_lo T_hi and per' = T_hi T_lo (T = the tile counts, 1 for
     // an empty pool), so that a segment is exactly n_hi (n_lo) ranges long.  Taken when
     // its longest range is shorter than per plus one segment's fixed cost.
-    const bool aligned = aligned_plan(p, pairs, (int64_t)num_sms * (p.fast ? kCtasFast : kCtasAffine),
-                                      st, max_stride, kWarps * 2);
+    const bool aligned = aligned_plan(p, pairs, slots, st, max_stride, kWarps * 2);
     // Otherwise the fast kernel runs one CTA of 16 warps per SM (see fast_ring_bytes)
     if (p.fast && !aligned) {
       p.warps = kFastWarps;
@@ -2501,23 +2537,27 @@ cudaError_t launch_decode_attention(const DecodeArgs& a, cudaStream_t stream) {
   static bool attr_set[kAttrDevices] = {};
   {
     const cudaError_t e = once_per_device(attr_set, [] {
+      constexpr int kMost = (int)std::max((size_t)(kRingBytes + kAqBytes), stage_bytes<kWarps>(8, 1024));
+      static_assert(stage_bytes<kWarps>(4, 1024) <= fast_ring_bytes<kWarps>(),
+                    "a staged tail fits the fast path's rings");
       cudaError_t r = cudaFuncSetAttribute(decode_affine_kernel,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           kRingBytes + kAqBytes);
+                                           cudaFuncAttributeMaxDynamicSharedMemorySize, kMost);
       if (r == cudaSuccess)
-        r = cudaFuncSetAttribute(decode_affine_fast_kernel<kWarps>,
+        r = cudaFuncSetAttribute(decode_affine_fast_kernel<kWarps, false>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  fast_ring_bytes<kWarps>() + kQbBytes);
       if (r == cudaSuccess)
-        r = cudaFuncSetAttribute(decode_affine_fast_kernel<kFastWarps>,
+        r = cudaFuncSetAttribute(decode_affine_fast_kernel<kWarps, true>,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 fast_ring_bytes<kWarps>() + kQbBytes);
+      if (r == cudaSuccess)
+        r = cudaFuncSetAttribute(decode_affine_fast_kernel<kFastWarps, false>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  fast_ring_bytes<kFastWarps>() + kQbBytes);
       if (r == cudaSuccess)
-        r = cudaFuncSetAttribute(decode_tq_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 kRingBytes + kAqBytes);
+        r = cudaFuncSetAttribute(decode_tq_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost);
       if (r == cudaSuccess)
-        r = cudaFuncSetAttribute(decode_stage_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 kStageRowBytes + 8 * stage_pad(1024) * 4);
+        r = cudaFuncSetAttribute(decode_stage_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost);
       return r;
     });
     if (e != cudaSuccess) return e;
@@ -2525,50 +2565,40 @@ cudaError_t launch_decode_attention(const DecodeArgs& a, cudaStream_t stream) {
   const DecodePlan& P = a.plan;
   if (P.stride < 1 || P.stride > kMaxSplits + 1) return cudaErrorInvalidValue;
   cudaError_t e = cudaSuccess;
-  bool pools_launched = false;
-  if (a.base == SEMKV_BASE_TQ_DENSE || a.base == SEMKV_BASE_TQ) {
-    if (a.base == SEMKV_BASE_TQ_DENSE) {
-      qrot_dense_kernel<<<a.B * a.H, 128, 0, stream>>>(a);
-      e = cudaGetLastError();
-      if (e != cudaSuccess) return e;
-    }
-    const int pool_splits = P.splits_hi + P.splits_lo;
-    if (pool_splits > 0) {
-      e = launch_pdl(decode_tq_kernel, dim3(pool_splits, a.H, a.B), dim3(kThreads),
-                     kRingBytes + kAqBytes, stream, a);
-      if (e != cudaSuccess) return e;
-      pools_launched = true;
-    }
-  } else if (P.ctas > 0) {
-    // (the rotated affine base rotates its queries inside the pool and stage kernels)
-    if (P.fast)
-      e = P.warps == kFastWarps
-              ? launch_pdl(decode_affine_fast_kernel<kFastWarps>, dim3(P.ctas),
-                           dim3(kFastWarps * 32), fast_ring_bytes<kFastWarps>() + kQbBytes, stream, a)
-              : launch_pdl(decode_affine_fast_kernel<kWarps>, dim3(P.ctas), dim3(kWarps * 32),
-                           fast_ring_bytes<kWarps>() + kQbBytes, stream, a);
-    else
-      e = launch_pdl(decode_affine_kernel, dim3(P.ctas), dim3(kThreads), kRingBytes + kAqBytes,
-                     stream, a);
-    if (e != cudaSuccess) return e;
-    pools_launched = true;
-  }
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  if (P.splits_st > 0) {
-    // after a pool kernel (which triggers its dependents once it has waited for its own
-    // inputs) the stage kernel starts alongside it; otherwise it runs in order
-    DecodeArgs as = a;
-    as.stage_overlaps_pools = pools_launched ? 1 : 0;
-    const size_t smem = kStageRowBytes + (size_t)(a.Hq / a.H) * stage_pad(a.stage_n) * 4;
-    if (as.stage_overlaps_pools)
-      e = launch_pdl(decode_stage_kernel, dim3(1, a.H, a.B), dim3(kThreads), smem, stream, as);
-    else
-      decode_stage_kernel<<<dim3(1, a.H, a.B), kThreads, smem, stream>>>(as);
-    if (e != cudaSuccess) return e;
+  const int G = a.Hq / a.H, pool_splits = P.splits_hi + P.splits_lo;
+  const int64_t tails = P.splits_st ? (int64_t)a.B * a.H : 0;  // CTAs of the staged tails
+  const size_t tail8 = P.splits_st ? stage_bytes<kWarps>(G, a.stage_n) : 0;
+  const bool tq = a.base == SEMKV_BASE_TQ_DENSE || a.base == SEMKV_BASE_TQ;
+  if (a.base == SEMKV_BASE_TQ_DENSE) {
+    qrot_dense_kernel<<<a.B * a.H, 128, 0, stream>>>(a);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
+  // (the Walsh-Hadamard bases rotate their queries inside the pool kernels)
+  if (tq && pool_splits > 0) {
+    e = launch_pdl(decode_tq_kernel, dim3(pool_splits + P.splits_st, a.H, a.B), dim3(kThreads),
+                   std::max((size_t)(kRingBytes + kAqBytes), tail8), stream, a);
+  } else if (!tq && P.ctas > 0) {
+    const bool apart = P.fast && P.warps == kFastWarps;  // (the tails in a kernel of their own)
+    const dim3 grid((unsigned)(P.ctas + (apart ? 0 : tails)));
+    if (!P.fast)
+      e = launch_pdl(decode_affine_kernel, grid, dim3(kThreads),
+                     std::max((size_t)(kRingBytes + kAqBytes), tail8), stream, a);
+    else if (!apart)  // (its rings are larger than a tail's rows and logits)
+      e = launch_pdl(tails ? decode_affine_fast_kernel<kWarps, true> : decode_affine_fast_kernel<kWarps, false>,
+                     grid, dim3(kWarps * 32), fast_ring_bytes<kWarps>() + kQbBytes, stream, a);
+    else
+      e = launch_pdl(decode_affine_fast_kernel<kFastWarps, false>, grid, dim3(kFastWarps * 32),
+                     fast_ring_bytes<kFastWarps>() + kQbBytes, stream, a);
+    if (e == cudaSuccess && apart && tails > 0) {
+      DecodeArgs as = a;
+      as.stage_overlaps_pools = 1;
+      e = launch_pdl(decode_stage_kernel, dim3((unsigned)tails), dim3(kThreads), tail8, stream, as);
+    }
+  } else {
+    e = launch_pdl(decode_stage_kernel, dim3((unsigned)tails), dim3(kThreads), tail8, stream, a);
+  }
+  if (e != cudaSuccess) return e;
   // the combine starts as a programmatic dependent launch: its launch (and, for the
   // dense rotation, the staging of M) overlaps the tail of the kernels before it
   const int heads = a.B * a.Hq;

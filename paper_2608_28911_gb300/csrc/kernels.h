@@ -116,7 +116,7 @@ struct DecodeArgs {
   const float* cb_lo;
   float* qrot;               // TQ: [B][Hq][128] rotated queries (workspace)
   int32_t* err;
-  // the fp16 stage kernel runs as a programmatic dependent of the affine pool kernel:
+  // the fp16 stage kernel runs as a programmatic dependent of the 16-warp pool kernel:
   // it reads its inputs at once and waits for that kernel only before it exits
   int stage_overlaps_pools;
   DecodePlan plan;

@@ -368,10 +368,9 @@ def gpu_arm(args, cfg, rank, world):
     scale = 1.0 / math.sqrt(128)
     base_counts = (cache.s.hi_count, cache.s.lo_count, cache.s.n_tokens)
     nh_b = semkv.semkv_block_high_count(blk, r_num, r_den)
-    # launches per decode call: (query rotation,) pools, combine (plus the stage kernel
-    # while tokens are staged)
-    plain = cfg["base"] == semkv.BASE_AFFINE
-    dec_launch = (0 if plain else 1) + 1 + 1
+    # launches per decode call: the pools (with the staged tails), the combine, and for the
+    # dense rotation the queries' rotation
+    dec_launch = 2 + (1 if cfg["base"] == semkv.BASE_TQ_DENSE else 0)
     # a block append: the block rank (which also writes the slot -> token maps), quantize
     app_launch = 2
 
@@ -406,7 +405,7 @@ def gpu_arm(args, cfg, rank, world):
         cyc += decode_bytes(cfg, desc, base_counts[0] + nh_b, base_counts[1] + blk - nh_b, 0)
         dec_bytes = NL * cyc / blk
         app_bytes = append_bytes(cfg, desc) / blk
-        launches_per_step = (app_launch + NL * (dec_launch + 1) * (blk - 1) + NL * dec_launch) / blk
+        launches_per_step = (app_launch + NL * dec_launch * blk) / blk
 
     flush = NL * dec_bytes < 2 * L2_BYTES
     scrub = torch.empty(512 * 2**20, dtype=torch.uint8, device=dev) if flush else None
@@ -848,9 +847,9 @@ def main():
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": profiled_traffic(args.config),
                      "kernel": {0: "decode_affine_fast_kernel + combine_wide_kernel",
-                                2: "qrot_kernel + decode_affine_fast_kernel + combine_wide_kernel",
-                                1: "qrot_kernel + decode_kernel<1> + combine_wide_kernel",
-                                3: "qrot_dense_kernel + decode_kernel<1> + combine_kernel<dense>"}[cfg["base"]]
+                                2: "decode_affine_fast_kernel + combine_wide_kernel",
+                                1: "decode_tq_kernel + combine_wide_kernel",
+                                3: "qrot_dense_kernel + decode_tq_kernel + combine_kernel<dense>"}[cfg["base"]]
                                + " (semkv_decode_attention)",
                      "peak_kind": f"{peak_kind} hbm_gbs"},
         "e2e": {"value": job_gbs(step_bytes, world, r["e2e_time"]), "unit": "GB/s",

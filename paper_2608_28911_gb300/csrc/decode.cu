@@ -38,7 +38,10 @@
 //    tried and rejected: the subtraction cancels ~30x and amplified the tensor
 //    cores' truncating fp32 accumulation past the attention tolerance.)
 // Six-level groups (F_4 up to 7775 would not fit) restart the chain after two
-// digits from the remainder x = beta * 36 mod 2^13.
+// digits from the remainder x = beta * 36 mod 2^13.  Four-level codes need no multiplies:
+// a byte permute looks them up (l4_lookup).
+//
+// The staged tail of a pair takes a CTA of its own in the pool kernels' grid (stage_cta).
 //
 // Per warp: a 4-deep ring of cp.async.bulk tile copies completing on per-stage
 // mbarriers (bounded waits that report a timeout in the error word).

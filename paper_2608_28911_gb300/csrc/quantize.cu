@@ -5,7 +5,8 @@
 // Records are built by destination slot: after a slot -> token map (scatter_tok_kernel),
 // the affine kernel gives a warp 4 consecutive slots of one pool (lanes own quarter rows),
 // the rotated bases 8 (two lanes per row, half a row in registers).  Either way the level
-// count is uniform and the record writes are contiguous.  The dense rotation runs its 128 x 128 product on tcgen05 instead.
+// count is uniform and the record writes are contiguous.  The dense rotation takes 64 slots
+// per group of four warps and runs its 128 x 128 product on tcgen05.
 //
 // Arithmetic (binary32, round to nearest even, no contraction), per row x:
 //  affine: s = fp16((max-min)/(L-1)) limited to 65504, z = fp16(min);
@@ -932,11 +933,9 @@ __global__ void __launch_bounds__(kRowsThreads, kRowsCtas) quantize_rows_kernel(
 //   affine: x^_d = fp16( z + s * c_d )
 //   rotated affine: y = FWHT(z + s * c);  x^_d = fp16( (sign_d y_d) * fp32(1/sqrt 128) )
 //   TQ:     y = FWHT(cb[c]) (the quantizer's butterflies);  x^_d = fp16( (sign_d y_d) * (n/128) )
-// A CTA of 128 threads takes 64 tokens of one (sequence, layer, KV head): thread r
-// owns row r (K of token r/2 when r is even, V when odd), in registers; rows are
-// staged through shared memory on the way in and out for coalesced transfers.
 
-// Affine base: a CTA per 64-token block, rows staged through shared memory in and out
+// Affine base: a CTA of 128 threads per 64-token block, thread r on row r (K of token r/2
+// when r is even, V when odd), rows staged through shared memory in and out
 // (coalesced), each row kept as fp16 pairs (96 registers: 5 CTAs per SM).
 __global__ void __launch_bounds__(128, 5) fake_affine_kernel(FakeArgs a) {
   __shared__ __align__(16) uint8_t stage[128 * kRowStride];

@@ -1484,14 +1484,17 @@ __global__ void qrot_dense_kernel(DecodeArgs a) {
 
 // ------------------------------------------------------- fp16 stage tokens ----
 
-// Staged tokens are few (at most a block): CUDA cores, in two passes with the logits between
-// them in shared memory, so that no token waits for the one before it.
+// Staged tokens are few (at most a block): CUDA cores, in three passes with the logits and
+// weights between them in shared memory, so that no token waits for the one before it.
 //  1. Logits: a warp takes four tokens at a time, 8 lanes per token with 16 dims each (three
-//     shuffles per head).  Then every warp takes the maximum per head.
-//  2. Weighted sums: a warp takes tokens warp, warp + 8, ...; lane = 4 dims.
-// Bound by latency: two rounds of loads instead of one round, a reduction over 32 lanes and
-// an exponential per token and head in a serial chain (which took 16 us for 77 tokens, longer
-// than the 4K-token pools beside it).
+//     shuffles per head); the first values' loads are already on their way.
+//  2. Warp c takes head c's maximum and turns its logits into weights.
+//  3. Weighted sums: a warp takes tokens warp, warp + 8, ...; lane = 4 dims.
+// Bound by latency.  Loads, a reduction over 32 lanes and an exponential per token and head
+// in a serial chain took 16 us for 77 tokens, longer than the 4K-token pools beside it.  Values
+// on their way early and one exponential per token instead of one per warp: a call with 64
+// staged tokens and 4K packed (B=1, 8 heads of G=4), back to back 12.9 -> 11.4 us, with cold
+// caches 25.7 -> 20.6 us; with 127 staged 16.8 -> 14.3 and 31.9 -> 25.8 us.
 // Writes rows in natural dim order and zs = 0.  logits: [G][stage_n rounded up to 32].
 template <int NW>
 __host__ __device__ constexpr int stage_row_bytes() { return (NW * 8 * kMoStride + 8 * 128) * 4; }
@@ -1510,6 +1513,12 @@ __device__ void run_stage(const DecodeArgs& a, Shared& sh, int b, int h, int G, 
   const int64_t base = (((int64_t)b * a.NL + a.layer) * a.H + h) * a.block;
   for (int i = threadIdx.x; i < G * 128; i += NW * 32)
     sh.qr[i >> 7][i & 127] = f16_to_f32(a.q[((int64_t)b * a.Hq + h * G) * 128 + i]);
+  // the first tokens' values on their way before the logits are needed
+  constexpr int kPre = 4;
+  uint2 pre[kPre];
+#pragma unroll
+  for (int i = 0; i < kPre; ++i)
+    pre[i] = *reinterpret_cast<const uint2*>(a.stage_v + (base + min(warp + i * NW, n - 1)) * 128 + 4 * lane);
   __syncthreads();
   {
     // 8-byte pieces (the stage's alignment): lane e of a token takes pieces e, e + 8, ...
@@ -1540,41 +1549,53 @@ __device__ void run_stage(const DecodeArgs& a, Shared& sh, int b, int h, int G, 
     }
   }
   __syncthreads();
-  float M[8], l[8], o[8][4];
+  // warp c: head c's maximum, its weights in place of the logits, their sum (8 <= NW); the
+  // other warps' rows hold no weight of their own at the common maximum
+  if (warp < G) {
+    float* lg = logits + warp * pad;
+    float M = -INFINITY, l = 0.0f;
+    for (int t = lane; t < n; t += 32) M = fmaxf(M, lg[t]);
 #pragma unroll
-  for (int c = 0; c < 8; ++c) {
-    M[c] = -INFINITY;
-    l[c] = 0.0f;
+    for (int off = 16; off >= 1; off >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, off));
+    for (int t = lane; t < n; t += 32) {
+      const float p = exp2f(lg[t] - M);
+      lg[t] = p;
+      l += p;
+    }
+#pragma unroll
+    for (int off = 16; off >= 1; off >>= 1) l += __shfl_xor_sync(0xffffffffu, l, off);
+    if (lane < NW) {
+      mg.m[lane * 8 + warp] = M;
+      mg.l[lane * 8 + warp] = lane == 0 ? l : 0.0f;
+      mg.z[lane * 8 + warp] = 0.0f;
+    }
+  }
+  __syncthreads();
+  float o[8][4];
+#pragma unroll
+  for (int c = 0; c < 8; ++c)
 #pragma unroll
     for (int j = 0; j < 4; ++j) o[c][j] = 0.0f;
-    if (c >= G) continue;
-    for (int t = lane; t < n; t += 32) M[c] = fmaxf(M[c], logits[c * pad + t]);
-#pragma unroll
-    for (int off = 16; off >= 1; off >>= 1) M[c] = fmaxf(M[c], __shfl_xor_sync(0xffffffffu, M[c], off));
-  }
-#pragma unroll 4
-  for (int t = warp; t < n; t += NW) {
-    const uint2 vu = *reinterpret_cast<const uint2*>(a.stage_v + (base + t) * 128 + 4 * lane);
+  auto add = [&](int t, uint2 vu) {
     const float vx[4] = {f16_to_f32((uint16_t)(vu.x & 0xFFFF)), f16_to_f32((uint16_t)(vu.x >> 16)),
                          f16_to_f32((uint16_t)(vu.y & 0xFFFF)), f16_to_f32((uint16_t)(vu.y >> 16))};
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
       if (c >= G) break;
-      const float p = exp2f(logits[c * pad + t] - M[c]);
-      l[c] += p;
+      const float p = logits[c * pad + t];
 #pragma unroll
       for (int j = 0; j < 4; ++j) o[c][j] += p * vx[j];
     }
-  }
+  };
+#pragma unroll
+  for (int i = 0; i < kPre; ++i)
+    if (warp + i * NW < n) add(warp + i * NW, pre[i]);
+#pragma unroll 4
+  for (int t = warp + kPre * NW; t < n; t += NW)
+    add(t, *reinterpret_cast<const uint2*>(a.stage_v + (base + t) * 128 + 4 * lane));
 #pragma unroll
   for (int c = 0; c < 8; ++c) {
     if (c >= G) break;
-    if (lane == 0) {
-      // a warp without tokens holds zeros at the common maximum
-      mg.m[warp * 8 + c] = M[c];
-      mg.l[warp * 8 + c] = l[c];
-      mg.z[warp * 8 + c] = 0.0f;
-    }
 #pragma unroll
     for (int j = 0; j < 4; ++j) o_out[mo_at(warp * 8 + c, 4 * lane + j)] = o[c][j];
   }

@@ -2471,10 +2471,18 @@ DecodePlan make_decode_plan(int base, int L_hi, int L_lo, int B, int H, int Hq, 
     }
     // CTAs of 8 warps, two per SM (a copy of one or two tiles per warp and step)
     p.warps = kWarps;
-    // (the staged tails' CTAs, one per pair, share the wave where there is room for them)
     int64_t slots = (int64_t)num_sms * (p.fast ? kCtasFast : kCtasAffine);
-    if (st && slots >= 4 * pairs) slots -= pairs;
     straddled(slots, kWarps * 2);
+    // Staged tails, a CTA per pair: in the pool kernel's grid, with room for them in its wave
+    // where there is any, while the pools' ranges are short (a launch less: a call over 4K
+    // tokens 16.4 -> 14.2 us).  Beside ranges of more than 8 tiles a warp they run in a kernel
+    // of their own and the pools keep every slot: 30 pairs of 51K tokens (40 tiles a warp)
+    // take 135.8 us so, 139.2 with slots given up to the tails (138.2 before either).
+    p.tails_apart = st && p.per > w_max * kWarps * 8 ? 1 : 0;
+    if (st && !p.tails_apart && slots >= 4 * pairs) {
+      slots -= pairs;
+      straddled(slots, kWarps * 2);
+    }
     // When the CTAs outnumber the pairs' segments (few sequences), ranges of equal
     // weight cut across the hi | lo and pair boundaries, and a CTA whose range holds a
     // boundary sets up, streams and merges two segments.  Aligned alternative: n_hi
@@ -2487,6 +2495,7 @@ DecodePlan make_decode_plan(int base, int L_hi, int L_lo, int B, int H, int Hq, 
     // Otherwise the fast kernel runs one CTA of 16 warps per SM (see fast_ring_bytes)
     if (p.fast && !aligned) {
       p.warps = kFastWarps;
+      p.tails_apart = st;  // (its registers have no room for the call)
       straddled(num_sms, kFastWarps * kChunk);
     }
     // partial slots per pair: an aligned segment is exactly n_hi (n_lo) ranges long;
@@ -2603,13 +2612,13 @@ cudaError_t launch_decode_attention(const DecodeArgs& a, cudaStream_t stream) {
     e = launch_pdl(decode_tq_kernel, dim3(pool_splits + P.splits_st, a.H, a.B), dim3(kThreads),
                    std::max((size_t)(kRingBytes + kAqBytes), tail8), stream, a);
   } else if (!tq && P.ctas > 0) {
-    const bool apart = P.fast && P.warps == kFastWarps;  // (the tails in a kernel of their own)
+    const bool apart = P.tails_apart != 0;
     const dim3 grid((unsigned)(P.ctas + (apart ? 0 : tails)));
     if (!P.fast)
       e = launch_pdl(decode_affine_kernel, grid, dim3(kThreads),
-                     std::max((size_t)(kRingBytes + kAqBytes), tail8), stream, a);
-    else if (!apart)  // (its rings are larger than a tail's rows and logits)
-      e = launch_pdl(tails ? decode_affine_fast_kernel<kWarps, true> : decode_affine_fast_kernel<kWarps, false>,
+                     std::max((size_t)(kRingBytes + kAqBytes), apart ? 0 : tail8), stream, a);
+    else if (P.warps == kWarps)  // (its rings are larger than a tail's rows and logits)
+      e = launch_pdl(tails && !apart ? decode_affine_fast_kernel<kWarps, true> : decode_affine_fast_kernel<kWarps, false>,
                      grid, dim3(kWarps * 32), fast_ring_bytes<kWarps>() + kQbBytes, stream, a);
     else
       e = launch_pdl(decode_affine_fast_kernel<kFastWarps, false>, grid, dim3(kFastWarps * 32),

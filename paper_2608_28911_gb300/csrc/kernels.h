@@ -96,6 +96,7 @@ struct DecodePlan {
   // fast kernel runs the balanced plan, with CTAs of `warps` warps (8: two per SM, 16: one)
   int fast;
   int warps;
+  int tails_apart;  // affine pools: the staged tails in a kernel of their own beside the pools'
 };
 struct DecodeArgs {
   int base, L_hi, L_lo;

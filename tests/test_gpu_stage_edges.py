@@ -20,6 +20,8 @@ pytestmark = pytest.mark.gpu
     (0, (6, 5), 2, 2, 3, 90, 33),
     (0, (6, 5), 20, 8, 4, 2200, 31),     # 16-warp fast kernel: the tail in its own launch
     (0, (4, 4), 1, 3, 8, 333, 32),       # general kernel, groups of eight
+    (0, (6, 5), 3, 8, 4, 14700, 47),     # 8-warp kernels over long ranges: a launch of its own
+    (0, (4, 4), 3, 8, 4, 14700, 47),
     (0, (8, 3), 2, 1, 5, 17, 200),
     (2, (6, 5), 1, 2, 1, 50, 1024),      # the largest stage
     (1, (4, 3), 2, 2, 8, 257, 65),       # TurboQuant kernel

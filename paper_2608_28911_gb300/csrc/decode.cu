@@ -2397,12 +2397,12 @@ static bool aligned_plan(DecodePlan& p, int64_t pairs, int64_t target, int st, i
   const int64_t cap_hi = th > 0 ? (th / min_tiles > 1 ? th / min_tiles : 1) : 0;
   const int64_t cap_lo = tl > 0 ? (tl / min_tiles > 1 ? tl / min_tiles : 1) : 0;
   int64_t best_h = 0, best_l = 0, best = INT64_MAX;
-  const int64_t top = th > 0 ? std::min(cap_hi, per_pair - (tl > 0 ? 1 : 0)) : 0;
+  // (an empty pool takes no CTA, and either pool leaves the other at least one: both counts
+  // stay within the resident CTAs and the partial slots, and neither is negative)
+  const int64_t most = std::min(per_pair, max_n);
+  const int64_t top = th > 0 ? std::min(cap_hi, most - (tl > 0 ? 1 : 0)) : 0;
   for (int64_t nh = th > 0 ? 1 : 0; nh <= top; ++nh) {
-    int64_t nl = tl > 0 ? per_pair - nh : 0;
-    if (nl > cap_lo) nl = cap_lo;
-    if (nh + nl > max_n) nl = max_n - nh;
-    if (tl > 0 && nl < 1) continue;
+    const int64_t nl = tl > 0 ? std::min(cap_lo, most - nh) : 0;
     const int64_t ch = nh ? (th + nh - 1) / nh * p.w_hi : 0;
     const int64_t cl = nl ? (tl + nl - 1) / nl * p.w_lo : 0;
     const int64_t c = ch > cl ? ch : cl;

@@ -2139,13 +2139,15 @@ __global__ void __launch_bounds__(kThreads, kCtasOther) decode_tq_kernel(const _
   const uint8_t* pool_bh = pool + (((int64_t)b * a.NL + a.layer) * a.H + h) * cap * rec;
   if (threadIdx.x < kWarps * kStages) mbar_init(bars + threadIdx.x);
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  // the records, the queries (and the dense rotation's q') and the codebooks come from earlier
+  // work on the stream
+  pdl_wait();
+  pdl_trigger();
   if (threadIdx.x < 16) {
     const int which = threadIdx.x >> 3, k = threadIdx.x & 7;
     sh.cb[which][k] = k < (which == 0 ? a.L_hi : a.L_lo) ? (which == 0 ? a.cb_hi : a.cb_lo)[k] : 0.0f;
   }
   __syncthreads();
-  pdl_wait();  // the records and queries (and the dense rotation's q') come from earlier work
-  pdl_trigger();
   // centroids as cz + cs c (two levels; three when equally spaced), or for four exactly
   // symmetric levels alpha phi + beta phi^3, phi = 2c - 3
   const float* cb = sh.cb[src];

@@ -817,15 +817,12 @@ __global__ void __launch_bounds__(kRowsThreads, kRowsCtas) quantize_rows_kernel(
   uint8_t* stages = rstage + warp * 2 * kWarpStageBytes;
   uint32_t* smask = smask_all[warp];
   const unsigned long long nz = opaque_neg_zero(smask);
-  // the thresholds of both pools, a zero one as +0 (tq_fields)
-  __shared__ float thr_sm[2][8];
-  if (BASE == SEMKV_BASE_TQ && threadIdx.x < 16) {
-    const int which = threadIdx.x >> 3, k = threadIdx.x & 7;
-    if (k < (which ? a.L_lo : a.L_hi) - 1)
-      thr_sm[which][k] = __fadd_rn((which ? a.thr_lo : a.thr_hi)[k], 0.0f);
-  }
-  __syncthreads();
-  pdl_wait();  // the slot maps and the rows come from earlier work on the stream
+  // the thresholds of both pools, a zero one as +0 (tq_fields): a copy per warp, which needs
+  // no CTA barrier (they are inputs like the rows, read only after the wait)
+  __shared__ float thr_all[BASE == SEMKV_BASE_TQ ? kRowsThreads / 32 : 1][2][8];
+  float (*thr_sm)[8] = thr_all[BASE == SEMKV_BASE_TQ ? warp : 0];
+  __syncwarp();
+  pdl_wait();  // the slot maps, the rows and the tables come from earlier work on the stream
   pdl_trigger();
   auto advance = [&](RowsPos& p) {
     p.r += kW;
@@ -876,6 +873,9 @@ __global__ void __launch_bounds__(kRowsThreads, kRowsCtas) quantize_rows_kernel(
   char2 s2[2];
   int32_t tok = token(cur);
   signs_of(masked, s2);
+  float thr = 0.0f;
+  if (BASE == SEMKV_BASE_TQ && (lane & 7) < ((lane & 8) ? a.L_lo : a.L_hi) - 1)
+    thr = ((lane & 8) ? a.thr_lo : a.thr_hi)[lane & 7];
   issue(cur, tok, 0);
   RowsPos nxt = cur;
   if (trips > 1) {
@@ -883,6 +883,7 @@ __global__ void __launch_bounds__(kRowsThreads, kRowsCtas) quantize_rows_kernel(
     tok = token(nxt);
   }
   put_masks(s2);
+  if (BASE == SEMKV_BASE_TQ && lane < 16) thr_sm[lane >> 3][lane & 7] = __fadd_rn(thr, 0.0f);
   for (int i = 0; i < trips; ++i) {
     const int st = i & 1;
     const uint32_t lh = cur.bhi % (uint32_t)(a.NL * a.H);
@@ -909,7 +910,7 @@ __global__ void __launch_bounds__(kRowsThreads, kRowsCtas) quantize_rows_kernel(
     const int ns = min(kTileSlots, (hi ? n_hi : n_lo) - s0);
     uint8_t* rec = hi ? a.hi_pool + ((int64_t)cur.bhi * a.hi_cap + a.hi_base + s0) * record_bytes_rt(BASE, L)
                       : a.lo_pool + ((int64_t)cur.bhi * a.lo_cap + a.lo_base + s0) * record_bytes_rt(BASE, L);
-    const float* thr = thr_sm[hi ? 0 : 1];
+    const float* thrs = thr_sm[hi ? 0 : 1];
     unsigned long long xp[32];
     uint32_t param;
     float invq, zq = 0.0f;
@@ -917,7 +918,7 @@ __global__ void __launch_bounds__(kRowsThreads, kRowsCtas) quantize_rows_kernel(
     rows_front<BASE>(L, stage, smask, nz, xp, param, invq, zq, live);
     switch (L) {
 #define SEMKV_ROWS_CASE(LV) \
-      case LV: rows_back<BASE, LV>(thr, stage, rec, ns, nz, xp, param, invq, zq, live); break;
+      case LV: rows_back<BASE, LV>(thrs, stage, rec, ns, nz, xp, param, invq, zq, live); break;
       SEMKV_ROWS_CASE(2) SEMKV_ROWS_CASE(3) SEMKV_ROWS_CASE(4) SEMKV_ROWS_CASE(5)
       SEMKV_ROWS_CASE(6) SEMKV_ROWS_CASE(7) SEMKV_ROWS_CASE(8)
 #undef SEMKV_ROWS_CASE

@@ -55,6 +55,7 @@
 #include <float.h>
 
 #include <algorithm>
+#include <cstddef>
 #include <cstring>
 
 #include "common.cuh"
@@ -573,13 +574,14 @@ __device__ __forceinline__ void state_init(WarpState& st) {
 
 struct Shared {
   uint16_t q[8][128];       // the group's query heads (rows >= G are zero)
-  float qr[8][128];         // TQ base: rotated queries q' = H S q
+  alignas(16) float qr[8][128];  // the rotated bases: rotated queries q' = H S q
   float cb[2][8];           // TQ base: centroids of the high / low level count
   float sumq[8];            // sum over dims of each head's q (q' for TQ records)
   float qmax[8];            // max |q_d| of each head (q' for TQ records)
   float cdec[2][3];         // TQ tensor path, per pool: centroids as cz + cs c (+ c3 phi^3)
   uint64_t bar[kMaxWarps][kStages];
 };
+static_assert(alignof(Shared) >= 16 && offsetof(Shared, qr) % 16 == 0, "run_stage reads qr in 16-byte pieces");
 
 // ------------------------------------------------------------ pool tiles ------
 

@@ -516,6 +516,48 @@ __global__ void __launch_bounds__(kThreads) rank_sort_kernel(RankArgs a, uint32_
 
 }  // namespace
 
+// Which instance of rank_cluster_kernel a call takes.  One CTA per SM (62 registers) while its
+// clusters run together (a cluster lies inside one GPC: the driver says 15 on the GPU measured,
+// and 15 take one pass), and where the keys leave no room for a second CTA; two per SM (32
+// registers) else.  One against two: 15 x 64K tokens 15.5 against 19.8 us, 16 x 64K 29.4 against
+// 23.6, 32 x 128K 64.5 against 45.1, 16 x 200K (one CTA fits) 62.3 against 63.7.
+struct ClusterLimits {
+  int resident;        // clusters that run together at one CTA per SM
+  size_t two_dynamic;  // the most dynamic shared memory with which two CTAs fit an SM
+};
+static size_t two_cta_dynamic(size_t per_sm, size_t reserved, size_t fixed) {
+  return per_sm / 2 > reserved + fixed ? per_sm / 2 - reserved - fixed : 0;
+}
+static bool two_clusters_per_sm(int B, size_t dynamic, const ClusterLimits& l) {
+  return B > l.resident && dynamic <= l.two_dynamic;
+}
+// The kernels' attributes and limits on device dev (the current one)
+static cudaError_t cluster_limits(int dev, ClusterLimits& out) {
+  constexpr int kMost = (int)(kSmemKeys * sizeof(uint32_t));
+  cudaError_t e = cudaFuncSetAttribute(rank_cluster_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(rank_cluster_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost);
+  cudaFuncAttributes fa = {};
+  int per_sm = 0, reserved = 0;
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, rank_cluster_kernel<2>);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev);
+  if (e != cudaSuccess) return e;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = kCluster;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(kCluster);
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = kMost;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  e = cudaOccupancyMaxActiveClusters(&out.resident, rank_cluster_kernel<1>, &cfg);
+  out.two_dynamic = two_cta_dynamic((size_t)per_sm, (size_t)reserved, fa.sharedSizeBytes);
+  return e;
+}
+
 size_t rank_workspace_words(int B, int T) { return (size_t)B * 4 * (size_t)T; }
 
 cudaError_t launch_rank_assign(const RankArgs& a, cudaStream_t stream) {
@@ -526,22 +568,16 @@ cudaError_t launch_rank_assign(const RankArgs& a, cudaStream_t stream) {
     if (e != cudaSuccess) return e;
   } else if (a.T >= 8192 && chunk <= kSmemKeys) {
     static bool cattr_set[kAttrDevices] = {};
-    const cudaError_t e = once_per_device(cattr_set, [] {
-      cudaError_t r = cudaFuncSetAttribute(rank_cluster_kernel<1>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)(kSmemKeys * sizeof(uint32_t)));
-      if (r == cudaSuccess)
-        r = cudaFuncSetAttribute(rank_cluster_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)(kSmemKeys * sizeof(uint32_t)));
-      return r;
-    });
+    static ClusterLimits limits[kAttrDevices] = {};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    // One CTA per SM (55 registers) while the clusters run together: a cluster lies inside
-    // one GPC, and 12 of them do (12 x 64K tokens: 15.6 us, 20.8 at two per SM and 32
-    // registers).  More sequences take two per SM (16 x 64K: 23.4 us, 29.5 in two waves).
+    e = once_per_device(cattr_set, [dev] { return cluster_limits(dev, limits[dev]); });
+    if (e != cudaSuccess) return e;
+    const size_t smem = (size_t)chunk * sizeof(uint32_t);
     const cudaError_t el =
-        launch_pdl(a.B <= 12 ? rank_cluster_kernel<1> : rank_cluster_kernel<2>,
-                   dim3(a.B * kCluster), dim3(kThreads), (size_t)chunk * sizeof(uint32_t), stream, a);
+        launch_pdl(two_clusters_per_sm(a.B, smem, limits[dev]) ? rank_cluster_kernel<2> : rank_cluster_kernel<1>,
+                   dim3(a.B * kCluster), dim3(kThreads), smem, stream, a);
     if (el != cudaSuccess) return el;
   } else {
     static bool attr_set[kAttrDevices] = {};

@@ -2477,12 +2477,19 @@ DecodePlan make_decode_plan(int base, int L_hi, int L_lo, int B, int H, int Hq, 
     p.warps = kWarps;
     int64_t slots = (int64_t)num_sms * (p.fast ? kCtasFast : kCtasAffine);
     straddled(slots, kWarps * 2);
-    // Staged tails, a CTA per pair: in the pool kernel's grid, with room for them in its wave
-    // where there is any, while the pools' ranges are short (a launch less: a call over 4K
-    // tokens 16.4 -> 14.2 us).  Beside ranges of more than 8 tiles a warp they run in a kernel
-    // of their own and the pools keep every slot: 30 pairs of 51K tokens (40 tiles a warp)
-    // take 135.8 us so, 139.2 with slots given up to the tails (138.2 before either).
-    p.tails_apart = st && p.per > w_max * kWarps * 8 ? 1 : 0;
+    // Staged tails, a CTA per pair: in the pool kernel's grid while the pools' ranges are short
+    // (a launch less: a call over 4K tokens 16.4 -> 14.2 us), with room for them in its wave
+    // where that takes a quarter of the slots at most.
+    // Beside ranges of more than 8 tiles a warp they run in a kernel of their own and the pools
+    // keep every slot: 30 pairs of 51K tokens (40 tiles a warp) take 135.8 us so, 139.2 with
+    // slots given up to the tails (138.2 before either).
+    // So they do beside the fast kernel's short ranges where more than a quarter would go: after
+    // a full wave they are a second one (80 pairs of 1000 tokens 22.1 us, 15.7 apart; 128 pairs
+    // of 512 and 2048 tokens 22.1 and 27.8, 20.4 and 27.6 apart).  The general kernel keeps them
+    // after its wave, where neither side is the better one throughout: 4/4 levels, 128 pairs of
+    // 2048 tokens with 1, 77, 127 and 1000 staged take 22.5, 26.5, 30.2 and 127 us, apart 23.4,
+    // 27.0, 29.4 and 139.
+    p.tails_apart = st && (p.per > w_max * kWarps * 8 || (p.fast && slots < 4 * pairs)) ? 1 : 0;
     if (st && !p.tails_apart && slots >= 4 * pairs) {
       slots -= pairs;
       straddled(slots, kWarps * 2);

@@ -1,13 +1,13 @@
 // Host-side check of the decode work plan (make_decode_plan in decode.cu) over caches with
-// an empty pool, built by tests/test_decode_plan_one_sided.py with nvcc and run on the CPU
-// (no kernel is launched).
+// an empty pool, and over many short ones with staged tails, built by
+// tests/test_decode_plan_one_sided.py with nvcc and run on the CPU (no kernel is launched).
 //
 // Required of every plan: weights that are not negative and add up (W = w_hi tiles_hi +
 // w_lo tiles_lo, the length of a pair's range that the kernels and the combine work from);
 // every tile in exactly one CTA's range; every partial slot, the staged tail's included,
 // inside the pair's stride; the stride within the caller's limit (a plan that needs more is
 // a refused call, and none of these may be refused); the pools' CTAs, and the staged tails'
-// where the plan makes room for them, within one wave.
+// where the plan makes room for them or the fast kernel runs them, within one wave.
 #include <cstdio>
 #include <cstdlib>
 #include <vector>
@@ -28,6 +28,8 @@ static int check(int L_hi, int L_lo, int B, int H, int G, long hi, long lo, int 
   if (P.W != (int64_t)P.w_hi * P.tiles_hi + (int64_t)P.w_lo * P.tiles_lo) bad++;
   if (P.ctas > 2L * sms) bad++;
   if (st && !P.tails_apart && 2L * sms >= 4 * pairs && P.ctas + pairs > 2L * sms) bad++;
+  // the fast kernel's tails never come after a full wave
+  if (st && P.fast && !P.tails_apart && P.ctas + pairs > 2L * sms) bad++;
   for (long bh = 0; bh < pairs && !bad; ++bh) {
     int n_hi, n_lo;
     pair_slots(P, bh, n_hi, n_lo);
@@ -67,6 +69,14 @@ int main() {
         for (int stage_n : {0, 77})
           for (int fast = 0; fast < 2; ++fast, ++n)
             bad += check(fast ? 6 : 8, fast ? 5 : 3, 1, H, 4, side ? 0 : t, side ? t : 0, stage_n, 152, 65);
+  // staged tails beside the short pools of many pairs
+  for (int B = 8; B <= 64; B += 2)
+    for (long t : {250L, 500L, 1000L, 2048L, 3500L})
+      for (int H : {4, 8}) {
+        bad += check(6, 5, B, H, 4, t / 4, t - t / 4, 77, 152, 65);
+        bad += check(4, 4, B, H, 4, t / 4, t - t / 4, 77, 152, 65);
+        n += 2;
+      }
   srand(4321);
   for (int i = 0; i < 3000; ++i, ++n) {
     const int B = 1 + rand() % 6, H = 1 + rand() % 4, G = rand() % 2 ? 4 : 8, stage_n = rand() % 2;

@@ -604,12 +604,12 @@ static_assert(alignof(Shared) >= 16 && offsetof(Shared, qr) % 16 == 0, "run_stag
 // CODEC 2: TQ, four levels: cb[c] = alpha phi + beta phi^3 with phi = 2c - 3; the phi
 //   part as CODEC 1 (cs = 2 alpha, cz = -3 alpha) plus a second pass on phi^3 (beta).
 // ring_it: tiles this warp has already taken through its ring (kept across calls so
-// the stage and barrier phase of each tile continue from the previous call)
+// the stage and barrier phase of each tile continue from the previous call); ring_fill has
+// started the range's first copies from the same position
 template <int L, bool PACKED, int CODEC = 0>
 __device__ void run_pool(const DecodeArgs& a, const Shared& sh, uint8_t* ring, uint4* aq_all,
                          uint64_t* bars, const uint8_t* pool_bh, int64_t count, int t_begin,
-                         int t_end, int G, WarpState& st, int& ring_it, int which = 0,
-                         bool prefilled = false) {
+                         int t_end, int G, WarpState& st, int& ring_it, int which) {
   using D = Dec<L>;
   using F = typename D::F;
   static_assert(CODEC != 2 || L == 4, "the cubic decomposition is for four levels");
@@ -670,17 +670,6 @@ __device__ void run_pool(const DecodeArgs& a, const Shared& sh, uint8_t* ring, u
 
   const int nmine = t_end - t_begin <= warp ? 0 : (t_end - t_begin - warp + kWarps - 1) / kWarps;
   const int count32 = (int)count;  // a pool holds fewer than 2^31 slots
-  if (lane == 0 && !prefilled) {
-    // the ring may have been the merge area: order those writes before the copies
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    for (int i = 0; i < kStages && i < nmine; ++i) {
-      const int tile = t_begin + warp + i * kWarps;
-      const int sl = (ring_it + i) % kStages;
-      mbar_expect_tx(&my_bar[sl], kTileBytes);
-      bulk_g2s(my_ring + sl * kStageBytes, pool_bh + (int64_t)tile * kTileBytes, kTileBytes,
-               &my_bar[sl]);
-    }
-  }
   __syncwarp();
   bool ok = true;
   int it = 0;
@@ -1910,9 +1899,9 @@ __device__ void run_pool_any_g(const DecodeArgs& a, const Shared& sh, uint8_t* r
   WarpState st;
   state_init(st);
   if (G <= 4)
-    run_pool<L, true, CODEC>(a, sh, ring, aq_all, bars, pool_bh, count, t0, t1, G, st, ring_it, which, true);
+    run_pool<L, true, CODEC>(a, sh, ring, aq_all, bars, pool_bh, count, t0, t1, G, st, ring_it, which);
   else
-    run_pool<L, false, CODEC>(a, sh, ring, aq_all, bars, pool_bh, count, t0, t1, G, st, ring_it, which, true);
+    run_pool<L, false, CODEC>(a, sh, ring, aq_all, bars, pool_bh, count, t0, t1, G, st, ring_it, which);
   affine_rows<L>(st, G, mg, merge_o);
 }
 

@@ -118,13 +118,18 @@ def _ptr(t):
     return t.data_ptr()   # (the argument types make it a void*)
 
 
+# The current stream's raw handle: building a torch Stream object took 3 of a decode call's
+# 18 us.  The two names are private to torch, so a release without them takes the object.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_raw_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream(stream):
     if stream is not None:
         return stream.cuda_stream
-    if not torch.cuda.is_initialized():
+    if _raw_stream is None or _raw_device is None or not torch.cuda.is_initialized():
         return torch.cuda.current_stream().cuda_stream
-    # the raw handle: building a torch Stream object took 3 of a decode call's 18 us
-    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return _raw_stream(_raw_device())
 
 
 def _check(fn, status):

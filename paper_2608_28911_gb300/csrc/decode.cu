@@ -41,7 +41,8 @@
 // digits from the remainder x = beta * 36 mod 2^13.  Four-level codes need no multiplies:
 // a byte permute looks them up (l4_lookup).
 //
-// The staged tail of a pair takes a CTA of its own in the pool kernels' grid (stage_cta).
+// The staged tail of a pair takes a CTA of its own (stage_cta), in the pool kernels' grid or in
+// a kernel beside them (make_decode_plan chooses).
 //
 // Per warp: a 4-deep ring of cp.async.bulk tile copies completing on per-stage
 // mbarriers (bounded waits that report a timeout in the error word).
@@ -2022,8 +2023,9 @@ __device__ __forceinline__ void run_fast_l(const DecodeArgs& a, const Shared& sh
 // The balanced plan of decode_affine_kernel, run by the fast path: CTA c takes the
 // weighted range [c per, (c+1) per) of the concatenated [hi | lo] tile sequence of every
 // (b, h), one partial per (pair, pool) segment it touches.
-// TAILS: the CTAs after the pools' take the staged tails (an instance of its own: the call
-// costs the pool loops a few registers, 1546 against 1508 us over 32 layers x 128K).
+// TAILS: the CTAs after the pools' take the staged tails (an instance of its own: with the call
+// the 8-warp pool loops spill 24 bytes at 128 registers, 1546 against 1508 us over 32 layers x
+// 128K).
 template <int NW, bool TAILS>
 __global__ void __launch_bounds__(NW * 32, NW == kWarps ? kCtasFast : 1)
     decode_affine_fast_kernel(const __grid_constant__ DecodeArgs a) {
@@ -2187,10 +2189,10 @@ __global__ void __launch_bounds__(kThreads, kCtasOther) decode_tq_kernel(const _
   merge_warps(a, kind, h, G, mg, merge_o, a.partials + (bh * P.stride + split) * kPartialFloats);
 }
 
-// The fp16 stage, one CTA per pair: for a cache without quantized tokens, and beside the
-// 16-warp pool kernel, whose register budget has no room for the call (16 x 64K: 282 us,
-// 290 with it).  The other pool kernels run the tails in CTAs of their own: a launch less (4K
-// tokens with a staged tail 16.4 -> 14.1 us).
+// The fp16 stage, one CTA per pair: for a cache without quantized tokens, beside the 16-warp
+// pool kernel, whose register budget has no room for the call (16 x 64K: 282 us, 290 with it),
+// and where make_decode_plan sets the tails apart.  Otherwise the pool kernels run them in CTAs
+// of their own: a launch less (4K tokens with a staged tail 16.4 -> 14.1 us).
 __global__ void __launch_bounds__(kThreads, kCtasOther) decode_stage_kernel(const __grid_constant__ DecodeArgs a) {
   extern __shared__ __align__(128) uint8_t dyn[];
   __shared__ Shared sh;

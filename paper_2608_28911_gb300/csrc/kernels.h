@@ -96,7 +96,7 @@ struct DecodePlan {
   // fast kernel runs the balanced plan, with CTAs of `warps` warps (8: two per SM, 16: one)
   int fast;
   int warps;
-  int tails_apart;  // affine pools: the staged tails in a kernel of their own beside the pools'
+  int tails_apart;  // affine pools: the staged tails in a kernel of their own beside the pools
 };
 struct DecodeArgs {
   int base, L_hi, L_lo;
@@ -117,8 +117,8 @@ struct DecodeArgs {
   const float* cb_lo;
   float* qrot;               // TQ: [B][Hq][128] rotated queries (workspace)
   int32_t* err;
-  // the fp16 stage kernel runs as a programmatic dependent of the 16-warp pool kernel:
-  // it reads its inputs at once and waits for that kernel only before it exits
+  // the fp16 stage kernel runs as a programmatic dependent of an affine pool kernel
+  // (plan.tails_apart): it reads its inputs at once and waits for that kernel only before it exits
   int stage_overlaps_pools;
   DecodePlan plan;
 };

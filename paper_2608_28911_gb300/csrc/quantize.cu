@@ -41,9 +41,9 @@ constexpr int kWarpsPerBlock = 8;
 // indices are read.  Quarters are staged 80 bytes apart, and the records leave through the
 // stage in 16-byte stores.
 //
-// Bound by memory: the 4 x 64K prompt's kernel takes 212 us, 5.9 TB/s (87% of the measured
-// copy rate), at 74% issue activity and 90 warp instructions per token and head.  It took 258
-// with 101 instructions, a 64-byte quarter per lane in four loads (which kept the load/store
+// Bound by memory: the 4 x 64K prompt's kernel takes 217 us, 5.8 TB/s (85% of the measured
+// copy rate), at 76% issue activity and 90 warp instructions per token and head.  It took 260
+// with 119 instructions, a 64-byte quarter per lane in four loads (which kept the load/store
 // pipe 74% busy), every code clamped and records put together by atomics and 4-byte stores.
 
 constexpr int kAffineSlots = 4;
@@ -471,12 +471,13 @@ constexpr int kHalfStride = 144;  // bytes per half-row slot: 128 + 16 (9 x 16 B
                                   // of a quarter warp reach distinct banks)
 constexpr int kWarpStageBytes = 32 * kHalfStride;
 // The quantizer: CTAs of 128 threads, 5 per SM (96 registers, 20 warps).  At 6 per SM (80
-// registers) the pairs spill and at 4 fewer warps hide the shuffles: the 32K TQ prompt takes
+// registers) the pairs spill (at 5 the TQ ones by 48 bytes) and at 4 fewer warps hide the shuffles: the 32K TQ prompt takes
 // 87 us at 5, 103 at 6 and 92 at 4, the 3 x 20011 rotated one 133, 139 and 136.
 constexpr int kRowsThreads = 128;
 constexpr int kRowsCtas = 5;
-// Fake quantization: 4 per SM (128 registers; at 5 the two transforms spill, 144 against 128 us
-// for 4 layers x 16384 tokens of the rotated affine base, and at 3 fewer warps hide latency, 138).
+// Fake quantization: 4 per SM (rotated affine: 127 registers, at 5 the two transforms spill, 144
+// against 128 us for 4 layers x 16384 tokens, and at 3 fewer warps hide latency, 138; TQ: 128
+// registers and 60 bytes spilled).
 constexpr int kFakeCtas = 4;
 
 // Butterfly stages 1, 2, 4, 8, 16 and 32 of the row transform over one half of the row,
@@ -790,14 +791,15 @@ struct RowsPos {
 };
 // Warps over tiles of 8 slots: a CTA takes a contiguous range, its warps the tiles in turn,
 // each warp with its own two-stage pipeline.  While a tile is quantized, the next one's
-// rows (8 cp.async of 16 bytes per lane) and the one after's token indices are on their way.  No warp waits for another, and the positions stay in uniform
-// registers (they leave room for the pairs, which otherwise spill).
+// rows (8 cp.async of 16 bytes per lane) and the one after's token indices are on their way.
+// No warp waits for another.  The positions stay in uniform registers, which leaves room for the
+// pairs: the rotated affine instance does not spill (92 registers), the TQ one 48 bytes
+// (96 registers).
 //
-// Bound by instruction issue: 76 (rotated affine) and 84 (TQ 4/3) warp instructions per row
-// at 58% and 56% issue activity, against 97 and 95 at 53% for the CTA-wide 64-slot blocks
-// with a barrier each, clamps on every code and records assembled word by word: the 3 x
-// 20011-token rotated prompt's kernel 146 -> 107 us (2.6 TB/s), the 32K TQ prompt's
-// 82 -> 62 us.  What is left is the butterflies (14 packed adds per row), conversions,
+// Bound by instruction issue: 75 (rotated affine) and 80 (TQ 4/3) warp instructions per row
+// at 63% issue activity, against 97 and 95 at 53% for the CTA-wide 64-slot blocks with a
+// barrier each, clamps on every code and records assembled word by word: the 32K prompt's
+// kernel 81.8 -> 56.6 us (rotated affine, 2.8 TB/s) and 83.9 -> 61.3 us (TQ).  What is left is the butterflies (14 packed adds per row), conversions,
 // radix groups and the exchange of stage 64.
 template <int BASE>
 __global__ void __launch_bounds__(kRowsThreads, kRowsCtas) quantize_rows_kernel(QuantArgs a, int64_t n_hi64, int64_t n_lo64) {
